@@ -179,8 +179,9 @@ struct RasClass {
   int local_off;      // offset of the class's packed local coordinates
   int nb;             // boxes per work item (batch width of the product)
   long long inv_off;  // offset of the inverse in the level's inverse array
-  int fdm_s[kMaxDim]; // fast diagonalisation: offset of each axis's sine matrix in the level's table
-  long long fdm_tri;  // fast diagonalisation: offset of the line-solve factors along the last axis
+  // fast diagonalisation in fixed point: offsets in the level's table of the
+  // transforms (forward, back) per axis and of the line-solve factors
+  int fx_f[2], fx_b[2], fx_tri;
 };
 
 struct Level {
@@ -215,7 +216,10 @@ struct Level {
   bool tc = false;                  // RAS products on the tensor cores (BF16 inverses)
   bool fdm = false;                 // FP64 local solves by fast diagonalisation and line solves
   int fdm_lmax = 0;                 // largest box extent along an axis (register bound of the kernel)
-  double* d_fdm = nullptr;          // sine matrices and line-solve factors of every class
+  int2* d_fix = nullptr;            // fixed-point sine matrices and line-solve factors of every class
+  int fx_zb = 0, fx_gb = 0;         // bits of the quantised iterate and right-hand side / of a residual alone
+  int fx_sf = 0, fx_kout = 0;       // exponent shifts of the right-hand side and of the results
+  int2 fx_kappa{};                  // stencil factor
   double fdm_flops = 0.0;           // algorithmic flops of one fast-diagonalisation smoothing product
   void* d_inv = nullptr;            // inverses in the W-cycle precision (row-major, symmetric)
   void* d_inv_bf16 = nullptr;       // optional BF16 copy
@@ -427,6 +431,10 @@ void mg_free(dcg_problem* p);
 int mg_inner_apply(dcg_problem* p, const double* z, double* y, cudaStream_t s);
 int mg_cycles(dcg_problem* p, const double* g, double* z, int ncycles, cudaStream_t s);
 int mg_solve(dcg_problem* p, const double* g, double* z, double tol, int nmax, int* ncyc, cudaStream_t s);
+// FP64 smoother's local solves in 64-bit fixed point (ras_fix.cu)
+int ras_fix_batch(int dim, int lmax);
+int ras_fix_setup(dcg_problem* p, Level& L, cudaStream_t s);
+int ras_fix_solve(dcg_problem* p, const Level& L, bool z_zero, cudaStream_t s);
 std::vector<int> level_sizes(int n, int max_levels);  // mesh sizes n_J, n_J/2, ... (finest first)
 int mg_ras_step_hook(dcg_problem* p, int level, const double* f, double* z, cudaStream_t s);
 // pieces of Algorithm 3 for the graph-captured solve (graph.cu)

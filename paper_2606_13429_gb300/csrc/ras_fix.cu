@@ -1,0 +1,749 @@
+// Exact local solves of the FP64 RAS smoother (Section 4.2) in 64-bit fixed
+// point, with the residual of the step formed in the same kernel.
+//
+// On a level whose stencil is the Q1 Laplacian / d (checked at setup), a
+// box's local matrix R_i Z_k R_i^T is (1/d) sum_i (x)_ax {K_l if ax = i else
+// M_l} with the 1D Dirichlet matrices K_l = (1/h) tridiag(-1, 2, -1) and
+// M_l = (h/6) tridiag(1, 4, 1) of the box extents l, both diagonalised by the
+// orthonormal sine matrix S_l. The exact solve (A_k)_i^{-1} r is then: S
+// along every axis but x, one tridiagonal solve per line along x (elimination
+// factors precomputed), S back.
+//
+// What bounds it. In FP64 the solve is bound by FP64 issue (2 lanes per
+// clock per SM): about 2,450 FP64 instructions per 12 x 12 box. The box data
+// therefore goes to fixed point (fix64.cuh), where a multiply-add costs three
+// integer multiply-adds on a pipe 32 times as wide; what is left is integer
+// issue (ALU pipe 57% busy: conversions, 64-bit additions and shifts beside
+// the multiply-adds) and the load phase. Measured per launch, residual
+// included: 2D 1024^2, 8 x 8 cores with overlap 2: 85.8 + 17.4 us (solve and
+// residual kernels in FP64) -> 50.0 us, 42.1 us from a zero iterate; 3D 128^3,
+// 4^3 cores with overlap 1: 270 + 99 us -> 163.6 us, 98.1 us. Against extended
+// precision a step's error falls from 1.1e-15 to 1.7e-16 of the result (2D,
+// 12 x 12 boxes, random data) and from 4.9e-16 to 2.8e-16 (3D).
+//
+// Scaling. All values of a box share one exponent, that of the largest of
+// |z| (box and its one-node halo) and |f| / hs (box), hs = 1 in 2D and the
+// power of two next below h in 3D, so that the scaled operator A / hs has
+// entries of order one whatever the level. Values are quantised to `zb` bits
+// (`gb` when the step starts from z = 0 and the residual is f itself); the
+// host chooses them from the row sums of the tables so that no intermediate
+// value can leave the range of fix64.cuh:
+//   residual growth, fold of two entries, transform |S|_inf, forward
+//   elimination, and the inverse line operators ||T_j^-1||_inf, which a
+//   transformed line j may grow by. In 2D line j is stored in units of
+//   2^K_j, K_j = ceil log2 ||T_j^-1||_inf, and the transform back multiplies
+//   by S 2^(K_j - kout); in 3D the growth is small and one K serves all.
+// A 12 x 12 box keeps 55 bits (57 from a zero iterate); an FP64 significand
+// has 53. A box with a non-finite entry returns NaN everywhere.
+//
+// Mapping. A CTA takes one work item (boxes of one class). In 2D a box belongs
+// to a group of 8, 16 or 32 lanes, one per column of the box and its halo: a
+// lane loads its column of z and f into registers (every load of the box in
+// flight together), the box maximum and the neighbouring columns come by
+// shuffles, the y transform runs down the lane's own column, the x line solve
+// takes one row per lane, and only the two transpositions between them go
+// through shared memory; no barrier wider than a warp. In 3D a box has one
+// thread per column along z (the perimeter columns of its halo are spread
+// over the same threads) and every phase gives each thread one grid line.
+// Rows are padded to an odd pitch (conflict-free 8-byte accesses).
+// A transform folds its line by the symmetry S[j][l-1-x] = (-1)^j S[j][x] (on
+// the inputs forward, on the outputs back): l^2 / 2 multiply-adds. Short
+// lines of a class are padded by zero table entries up to the compile-time
+// LM. Results go to y box-major (y[item][b][i]).
+#include "common.cuh"
+#include "fix64.cuh"
+
+#include <algorithm>
+#include <cmath>
+#include <map>
+#include <utility>
+
+namespace dcg {
+namespace {
+
+struct FixArgs {
+  const int* work;           // [nwork*3]: class, first index into class_patches, count
+  const int* class_patches;
+  const RasClass* classes;
+  const int4* origin;        // [npatch] box origin (x, y, z) and its node index
+  const long long* item_off; // [nwork]
+  const int2* tab;
+  int m, bits, sf, kout;     // bits: zb or gb; f is scaled by 2^sf
+  int2 kappa;                // r = f 2^sf + kappa T(z), T the integer stencil sum
+};
+
+constexpr int fx_group(int LM) { return LM + 2 <= 8 ? 8 : LM + 2 <= 16 ? 16 : 32; }  // lanes per box, 2D
+constexpr int fx_batch(int D, int LM) { return D == 2 ? 128 / fx_group(LM) : 8; }
+constexpr int fx_threads(int D, int LM) { return D == 2 ? 128 : 8 * LM * LM; }
+// CTAs per SM the register allocation leaves room for
+constexpr int fx_blocks(int D, int LM) { return D == 2 ? (LM <= 8 ? 7 : LM <= 12 ? 6 : 4) : (LM <= 4 ? 6 : 2); }
+// pitch of a line of table constants (pairs are read as 16-byte loads)
+__host__ __device__ constexpr int fx_hm(int LM) { return ((LM + 1) / 2 + 1) / 2 * 2; }
+
+// forward transform of one line in place; C[j][x], x < fx_hm(LM)
+template <int LM>
+__device__ __forceinline__ void fx_forward(long long* __restrict__ W, int stride, int l, const int2* __restrict__ C) {
+  constexpr int HM = (LM + 1) / 2, HP = fx_hm(LM);
+  const int h = l >> 1, hc = (l + 1) >> 1;
+  FxVal p[HP], q[HP];
+#pragma unroll
+  for (int x = 0; x < HP; ++x) {
+    const long long a = (x < HM && x < hc) ? W[x * stride] : 0;
+    const long long b = (x < HM && x < h) ? W[(l - 1 - x) * stride] : 0;
+    p[x] = fx_split(a + b);
+    q[x] = fx_split(a - b);
+  }
+  // two outputs per turn of a rolled loop: unrolled, the table loads of many
+  // outputs are hoisted together and take 250 registers
+#pragma unroll 1
+  for (int j = 0; j < l; j += 2) {
+    FxAcc e = fx_zero(), o = fx_zero();
+#pragma unroll
+    for (int x = 0; x < HP; x += 2) {
+      const int4 ce = *reinterpret_cast<const int4*>(C + j * HP + x);
+      const int4 co = *reinterpret_cast<const int4*>(C + (j + 1) * HP + x);
+      fx_mac(e, p[x], ce.x, ce.y);
+      fx_mac(o, q[x], co.x, co.y);
+      if (x + 1 < HM) {
+        fx_mac(e, p[x + 1], ce.z, ce.w);
+        fx_mac(o, q[x + 1], co.z, co.w);
+      }
+    }
+    W[j * stride] = fx_value(e);
+    if (j + 1 < l) W[(j + 1) * stride] = fx_value(o);
+  }
+}
+
+// transform back: out_x = sum_j C_x[j] v_j; C[x][j], x < (LM+1)/2, j < LM
+// (even j, then odd j, each padded to fx_hm(LM))
+template <int LM>
+__device__ __forceinline__ void fx_back(long long* __restrict__ W, int stride, int l, const int2* __restrict__ C) {
+  constexpr int HM = (LM + 1) / 2, HP = fx_hm(LM);
+  const int h = l >> 1, hc = (l + 1) >> 1;
+  FxVal v[2 * HP];
+#pragma unroll
+  for (int j = 0; j < 2 * HP; ++j) v[j] = fx_split((j < LM && j < l) ? W[j * stride] : 0);
+#pragma unroll 1
+  for (int x = 0; x < hc; ++x) {
+    FxAcc e = fx_zero(), o = fx_zero();
+#pragma unroll
+    for (int k = 0; k < HP; k += 2) {
+      const int4 ce = *reinterpret_cast<const int4*>(C + (2 * x) * HP + k);
+      const int4 co = *reinterpret_cast<const int4*>(C + (2 * x + 1) * HP + k);
+      fx_mac(e, v[2 * k], ce.x, ce.y);
+      fx_mac(o, v[2 * k + 1], co.x, co.y);
+      if (k + 1 < HM) {
+        fx_mac(e, v[2 * k + 2], ce.z, ce.w);
+        fx_mac(o, v[2 * k + 3], co.z, co.w);
+      }
+    }
+    const long long E = fx_value(e), O = fx_value(o);
+    W[x * stride] = E + O;
+    if (x < h) W[(l - 1 - x) * stride] = E - O;
+  }
+}
+
+// line solve in place. t: [4][n][nl] constants of this line with pitch nl:
+// -l_i; winv_i 2^-K; -b winv_i; and, for the exact extent n = LM, in entry
+// [3][0] the reciprocal pivot of the meeting row.
+// General extents: y_i = g_i - l_i y_{i-1}; x_i = winv_i y_i - b winv_i x_{i+1}.
+// n = LM: the line is Toeplitz, so it is eliminated from both ends with the
+// same factors, the two chains meeting at rows LM/2 - 1 and LM/2 (half the
+// dependent steps).
+template <int LM, bool EX>
+__device__ __forceinline__ void fx_line_solve(long long* __restrict__ W, int n, const int2* __restrict__ t, int nl) {
+  long long g[LM];
+#pragma unroll
+  for (int i = 0; i < LM; ++i) g[i] = (EX || i < n) ? W[i] : 0;
+  if constexpr (EX) {
+    constexpr int H = LM / 2;
+#pragma unroll
+    for (int i = 1; i < H; ++i) {
+      const int2 c = __ldg(t + i * nl);
+      FxAcc a = fx_zero(), d = fx_zero();
+      fx_mac(a, fx_split(g[i - 1]), c.x, c.y);
+      fx_mac(d, fx_split(g[LM - i]), c.x, c.y);
+      g[i] += fx_value(a);
+      g[LM - 1 - i] += fx_value(d);
+    }
+    // row H with the whole upper half eliminated
+    long long xa, xb;
+    {
+      const int2 c = __ldg(t + H * nl), cm = __ldg(t + 3 * LM * nl);
+      FxAcc a = fx_zero(), d = fx_zero();
+      fx_mac(a, fx_split(g[H - 1]), c.x, c.y);
+      fx_mac(d, fx_split(g[H] + fx_value(a)), cm.x, cm.y);
+      xb = fx_value(d);
+      W[H] = xb;
+    }
+    {
+      const int2 cw = __ldg(t + (LM + H - 1) * nl), cb = __ldg(t + (2 * LM + H - 1) * nl);
+      FxAcc a = fx_zero();
+      fx_mac(a, fx_split(g[H - 1]), cw.x, cw.y);
+      fx_mac(a, fx_split(xb), cb.x, cb.y);
+      xa = fx_value(a);
+      W[H - 1] = xa;
+    }
+#pragma unroll
+    for (int i = H - 2; i >= 0; --i) {
+      const int2 cw = __ldg(t + (LM + i) * nl), cb = __ldg(t + (2 * LM + i) * nl);
+      FxAcc a = fx_zero(), d = fx_zero();
+      fx_mac(a, fx_split(g[i]), cw.x, cw.y);
+      fx_mac(d, fx_split(g[LM - 1 - i]), cw.x, cw.y);
+      fx_mac(a, fx_split(xa), cb.x, cb.y);
+      fx_mac(d, fx_split(xb), cb.x, cb.y);
+      xa = fx_value(a);
+      xb = fx_value(d);
+      W[i] = xa;
+      W[LM - 1 - i] = xb;
+    }
+  } else {
+#pragma unroll
+    for (int i = 1; i < LM; ++i)
+      if (i < n) {
+        const int2 c = __ldg(t + i * nl);
+        FxAcc a = fx_zero();
+        fx_mac(a, fx_split(g[i - 1]), c.x, c.y);
+        g[i] += fx_value(a);
+      }
+    long long xn = 0;
+#pragma unroll
+    for (int i = LM - 1; i >= 0; --i)
+      if (i < n) {
+        const int2 cw = __ldg(t + (n + i) * nl), cb = __ldg(t + (2 * n + i) * nl);
+        FxAcc a = fx_zero();
+        fx_mac(a, fx_split(g[i]), cw.x, cw.y);
+        fx_mac(a, fx_split(xn), cb.x, cb.y);
+        xn = fx_value(a);
+        W[i] = xn;
+      }
+  }
+}
+
+// result of a box that is all zero, has a non-finite entry, or may overflow
+__device__ __forceinline__ double fx_special(long long v, int e0, unsigned mag) {
+  if (mag == 0) return 0.0;
+  return mag < kFxNonFinite ? fx_to_double(v, e0, false) : __longlong_as_double(0x7ff8000000000000ll);
+}
+
+// EX: the boxes have extent LM along every axis
+template <int LM, bool ZZERO, bool EX>
+__device__ __forceinline__ void fx_boxes_2d(const FixArgs& A, const RasClass& C, const int2* s_tab, long long* smem,
+                                            int first, int cnt, const double* __restrict__ f,
+                                            const double* __restrict__ z, double* __restrict__ yi) {
+  constexpr int G = fx_group(LM), HP = fx_hm(LM), NF = LM * HP;
+  const int lane = threadIdx.x & (G - 1), b = threadIdx.x / G;
+  const int lx = EX ? LM : C.len[0], ly = EX ? LM : C.len[1], m = A.m;
+  const int wp = lx | 1;                     // row pitch of the box values
+  long long* W = smem + b * (ly * wp);       // [ly][wp]
+  const bool live = b < cnt;                 // groups past the item's boxes only take part in the shuffles
+  const int x = lane - 1;                    // column of the box, -1 and lx are its halo
+  const bool own = live && x >= 0 && x < lx;
+  const int4 og = live ? __ldg(A.origin + __ldg(A.class_patches + first + b)) : make_int4(0, 0, 0, 0);
+  long long zv[LM + 2], fv[LM];
+  {
+    const int gx = og.x + x;
+    const bool col = live && !ZZERO && x <= lx && gx >= 0 && gx < m;
+    const int base = gx + m * (og.y - 1);
+#pragma unroll
+    for (int q = 0; q < LM + 2; ++q) {
+      const int gy = og.y - 1 + q;
+      // rows 1 .. ly of the halo lie in the box and so in the grid
+      zv[q] = (col && q <= ly + 1 && (EX && q >= 1 && q <= LM ? true : gy >= 0 && gy < m)) ? __double_as_longlong(__ldg(z + base + q * m)) : 0;
+    }
+#pragma unroll
+    for (int q = 0; q < LM; ++q)
+      fv[q] = (own && q < ly) ? __double_as_longlong(__ldg(f + base + (q + 1) * m)) : 0;
+  }
+  unsigned mag = 0;
+#pragma unroll
+  for (int q = 0; q < LM; ++q) mag = max(mag, fx_mag(fv[q]));
+  if (!ZZERO) {
+#pragma unroll
+    for (int q = 0; q < LM + 2; ++q) mag = max(mag, fx_mag(zv[q]));
+  }
+#pragma unroll
+  for (int o = G / 2; o > 0; o >>= 1) mag = max(mag, __shfl_xor_sync(0xffffffffu, mag, o, G));
+  const int e = fx_block_exponent(mag), sh0 = 63 - A.bits + e;
+  // residual r = f + kappa T(z), T = (sum of the 3 x 3 box) - 9 z
+  if (ZZERO) {
+#pragma unroll
+    for (int q = 0; q < LM; ++q)
+      if (own && q < ly) W[q * wp + x] = fx_near(fv[q], sh0);
+  } else {
+    long long s0 = 0, s1 = 0, zm = 0;
+#pragma unroll
+    for (int q = 0; q < LM + 2; ++q) {
+      const long long zc = fx_floor(zv[q], sh0);
+      const long long s2 = __shfl_up_sync(0xffffffffu, zc, 1, G) + zc + __shfl_down_sync(0xffffffffu, zc, 1, G);
+      if (q >= 2) {
+        const long long T = (s0 + s1 + s2) - (zm << 3) - zm;
+        FxAcc a = fx_zero();
+        fx_mac(a, fx_split(T), A.kappa.x, A.kappa.y);
+        if (own && q - 2 < ly) W[(q - 2) * wp + x] = fx_near(fv[q - 2], sh0) + fx_value(a);
+      }
+      s0 = s1;
+      s1 = s2;
+      zm = zc;
+    }
+  }
+  if (own) fx_forward<LM>(W + x, wp, ly, s_tab);
+  __syncwarp();
+  if (live && lane < ly) fx_line_solve<LM, EX>(W + lane * wp, lx, A.tab + C.fx_tri + lane, ly);
+  __syncwarp();
+  if (own) {
+    fx_back<LM>(W + x, wp, ly, s_tab + NF);
+    const int e0 = e + 63 - A.bits + A.kout;
+    const bool safe = mag != 0 && mag < kFxNonFinite && e0 < 0x7ff;
+    double* yb = yi + b * (lx * ly) + x;
+    if (safe) {
+#pragma unroll 4
+      for (int q = 0; q < ly; ++q) yb[q * lx] = fx_to_double(W[q * wp + x], e0, true);
+    } else {
+      for (int q = 0; q < ly; ++q) yb[q * lx] = fx_special(W[q * wp + x], e0, mag);
+    }
+  }
+}
+
+template <int LM, bool ZZERO, bool EX>
+__device__ __forceinline__ void fx_boxes_3d(const FixArgs& A, const RasClass& C, const int2* s_tab, long long* smem, unsigned* s_e,
+                                            int first, int cnt, const double* __restrict__ f,
+                                            const double* __restrict__ z, double* __restrict__ yi) {
+  constexpr int TPB = LM * LM, HP = fx_hm(LM), HM = (LM + 1) / 2, NF = LM * HP, NBK = 2 * HM * HP;
+  constexpr int NB = fx_batch(3, LM);
+  constexpr int PE = (4 * LM + 4 + TPB - 1) / TPB;  // perimeter columns per thread
+  const int b = threadIdx.x / TPB, c = threadIdx.x - b * TPB;
+  const int cy = c / LM, cx = c - cy * LM;
+  const int lx = EX ? LM : C.len[0], ly = EX ? LM : C.len[1], lz = EX ? LM : C.len[2], m = A.m;
+  const int wp = lx | 1, hx = lx + 2, hy = ly + 2;
+  const int wb = wp * ly * lz, zn = hx * hy * (lz + 2);
+  long long* W = smem + b * wb;              // [lz][ly][wp]
+  long long* Z = smem + NB * wb + b * zn;    // [lz + 2][hy][hx]
+  const bool live = b < cnt;
+  const bool own = live && cx < lx && cy < ly;
+  const int4 og = live ? __ldg(A.origin + __ldg(A.class_patches + first + b)) : make_int4(0, 0, 0, 0);
+  if (c == 0) s_e[b] = 0;
+  __syncthreads();
+  const int mm = m * m;
+  long long zv[LM + 2], fv[LM], pv[PE][LM + 2];
+  int px[PE], py[PE];
+  unsigned mag = 0;
+  {
+    const int base = (og.x + cx) + m * (og.y + cy) + mm * (og.z - 1);
+#pragma unroll
+    for (int q = 0; q < LM; ++q) {
+      fv[q] = (own && q < lz) ? __double_as_longlong(__ldg(f + base + (q + 1) * mm)) : 0;
+      const unsigned mf = fx_mag(fv[q]);
+      mag = max(mag, mf >= kFxNonFinite || mf == 0 ? mf : (unsigned)max((int)mf + (A.sf << 20), 1));
+    }
+    if (!ZZERO) {
+#pragma unroll
+      for (int q = 0; q < LM + 2; ++q) {
+        const int gz = og.z - 1 + q;
+        zv[q] = (own && q <= lz + 1 && gz >= 0 && gz < m) ? __double_as_longlong(__ldg(z + base + q * mm)) : 0;
+        mag = max(mag, fx_mag(zv[q]));
+      }
+#pragma unroll
+      for (int k = 0; k < PE; ++k) {
+        // perimeter column t of the halo: the rows y = -1 and y = ly, then
+        // the sides x = -1, lx
+        const int t = c + k * TPB, u = t - 2 * hx;
+        px[k] = t < hx ? t : t < 2 * hx ? t - hx : (u & 1) ? hx - 1 : 0;
+        py[k] = t < hx ? 0 : t < 2 * hx ? hy - 1 : 1 + (u >> 1);
+        const int gx = og.x - 1 + px[k], gy = og.y - 1 + py[k];
+        const bool per = live && t < 2 * hx + 2 * ly;
+        const bool col = per && gx >= 0 && gx < m && gy >= 0 && gy < m;
+        const int pb = gx + m * gy + mm * (og.z - 1);
+#pragma unroll
+        for (int q = 0; q < LM + 2; ++q) {
+          const int gz = og.z - 1 + q;
+          pv[k][q] = (col && q <= lz + 1 && gz >= 0 && gz < m) ? __double_as_longlong(__ldg(z + pb + q * mm)) : 0;
+          mag = max(mag, fx_mag(pv[k][q]));
+        }
+        if (!per) px[k] = -1;
+      }
+    }
+  }
+  if (live && mag) atomicMax(&s_e[b], mag);
+  __syncthreads();
+  mag = s_e[b];
+  const int e = fx_block_exponent(mag), sh0 = 63 - A.bits + e;
+  if (ZZERO) {
+#pragma unroll
+    for (int q = 0; q < LM; ++q)
+      if (own && q < lz) W[(q * ly + cy) * wp + cx] = fx_near(fv[q], sh0 - A.sf);
+  } else {
+#pragma unroll
+    for (int q = 0; q < LM + 2; ++q) {
+      zv[q] = fx_floor(zv[q], sh0);
+      if (own && q <= lz + 1) Z[(q * hy + cy + 1) * hx + cx + 1] = zv[q];
+#pragma unroll
+      for (int k = 0; k < PE; ++k)
+        if (px[k] >= 0 && q <= lz + 1) Z[(q * hy + py[k]) * hx + px[k]] = fx_floor(pv[k][q], sh0);
+    }
+    __syncthreads();
+    // T = S3 + 2 S2 - 32 z (S2 the 12 edge, S3 the 8 corner neighbours; the 6
+    // face coefficients of the 3D Q1 Laplacian vanish)
+    if (own) {
+      long long Em = 0, E0 = 0, D0 = 0;
+#pragma unroll
+      for (int q = 0; q < LM + 2; ++q) {
+        const long long* p = Z + (min(q, lz + 1) * hy + cy) * hx + cx;  // planes past lz + 1 are not used
+        const long long D4 = (p[0] + p[2]) + (p[2 * hx] + p[2 * hx + 2]);
+        const long long Ep = D4 + ((p[hx] + p[hx + 2] + p[1] + p[2 * hx + 1]) << 1);
+        if (q >= 2) {
+          const long long T = Em + Ep + (D0 << 1) - (zv[q - 1] << 5);
+          FxAcc a = fx_zero();
+          fx_mac(a, fx_split(T), A.kappa.x, A.kappa.y);
+          if (q - 2 < lz) W[((q - 2) * ly + cy) * wp + cx] = fx_near(fv[q - 2], sh0 - A.sf) + fx_value(a);
+        }
+        Em = E0;
+        E0 = Ep;
+        D0 = D4;
+      }
+    }
+  }
+  // column (cx, cy) along z; then line (cx, k = cy) along y; then line (j =
+  // cx, k = cy) along x
+  if (own) fx_forward<LM>(W + cy * wp + cx, ly * wp, lz, s_tab + NF + NBK);
+  __syncthreads();
+  const bool yline = live && cx < lx && cy < lz;
+  if (yline) fx_forward<LM>(W + cy * ly * wp + cx, wp, ly, s_tab);
+  __syncthreads();
+  if (live && cx < ly && cy < lz)
+    fx_line_solve<LM, EX>(W + (cy * ly + cx) * wp, lx, A.tab + C.fx_tri + cy * ly + cx, ly * lz);
+  __syncthreads();
+  if (yline) fx_back<LM>(W + cy * ly * wp + cx, wp, ly, s_tab + NF);
+  __syncthreads();
+  if (own) {
+    fx_back<LM>(W + cy * wp + cx, ly * wp, lz, s_tab + NF + NBK + NF);
+    const int e0 = e + 63 - A.bits + A.kout;
+    const bool safe = mag != 0 && mag < kFxNonFinite && e0 < 0x7ff;
+    double* yb = yi + b * (lx * ly * lz) + cy * lx + cx;
+    if (safe) {
+#pragma unroll 2
+      for (int q = 0; q < lz; ++q) yb[q * lx * ly] = fx_to_double(W[(q * ly + cy) * wp + cx], e0, true);
+    } else {
+      for (int q = 0; q < lz; ++q) yb[q * lx * ly] = fx_special(W[(q * ly + cy) * wp + cx], e0, mag);
+    }
+  }
+}
+
+template <int D, int LM, bool ZZERO>
+__global__ void __launch_bounds__(fx_threads(D, LM), fx_blocks(D, LM))
+    k_ras_fix(FixArgs A, const double* __restrict__ f, const double* __restrict__ z, double* __restrict__ y) {
+  constexpr int HP = fx_hm(LM), HM = (LM + 1) / 2;
+  constexpr int NF = LM * HP, NBK = 2 * HM * HP;  // forward / back table entries per axis
+  extern __shared__ __align__(16) unsigned char fx_smem[];
+  __shared__ __align__(16) int2 s_tab[(D - 1) * (NF + NBK)];
+  __shared__ unsigned s_e[fx_batch(D, LM)];
+  const int w = blockIdx.x;
+  const int cls = A.work[3 * w], first = A.work[3 * w + 1], cnt = A.work[3 * w + 2];
+  const RasClass& C = A.classes[cls];
+  for (int t = threadIdx.x; t < (D - 1) * (NF + NBK); t += fx_threads(D, LM)) {
+    const int ax = t / (NF + NBK), i = t - ax * (NF + NBK);
+    s_tab[t] = __ldg(A.tab + (i < NF ? C.fx_f[ax] + i : C.fx_b[ax] + i - NF));
+  }
+  __syncthreads();
+  long long* smem = reinterpret_cast<long long*>(fx_smem);
+  double* yi = y + A.item_off[w];
+  const bool exact = C.len[0] == LM && C.len[1] == LM && (D == 2 || C.len[2] == LM);  // the interior class
+  if constexpr (D == 2) {
+    if (exact) fx_boxes_2d<LM, ZZERO, true>(A, C, s_tab, smem, first, cnt, f, z, yi);
+    else fx_boxes_2d<LM, ZZERO, false>(A, C, s_tab, smem, first, cnt, f, z, yi);
+  } else {
+    if (exact) fx_boxes_3d<LM, ZZERO, true>(A, C, s_tab, smem, s_e, first, cnt, f, z, yi);
+    else fx_boxes_3d<LM, ZZERO, false>(A, C, s_tab, smem, s_e, first, cnt, f, z, yi);
+  }
+}
+
+long long fx_const_bits(long double c) { return (long long)llroundl(c * 288230376151711744.0L); }  // 2^58
+// the constant C 2^-58 2^shift as the pair fx_mac takes
+int2 fx_const(long long C, int shift = 0) {
+  const long long v = shift >= 0 ? C << shift : (C + (1LL << (-shift - 1))) >> -shift;
+  const long long lo = ((v + (1LL << 28)) & ((1LL << 29) - 1)) - (1LL << 28);  // in [-2^28, 2^28)
+  return make_int2((int)((v - lo) >> 29), (int)lo);
+}
+
+template <int D, int LM>
+size_t fx_smem(const Level& L) {
+  size_t mx = 0;
+  for (const auto& c : L.classes) {
+    const size_t wb = (size_t)(c.len[0] | 1) * c.len[1] * (D > 2 ? c.len[2] : 1);
+    const size_t zn = D > 2 ? (size_t)(c.len[0] + 2) * (c.len[1] + 2) * (c.len[2] + 2) : 0;
+    mx = std::max(mx, sizeof(long long) * (size_t)c.nb * (wb + zn));
+  }
+  return mx;
+}
+
+template <int D, int LM>
+int fx_attr(const Level& L) {
+  const int smem = (int)fx_smem<D, LM>(L);
+  DCG_CUDA(cudaFuncSetAttribute(k_ras_fix<D, LM, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  DCG_CUDA(cudaFuncSetAttribute(k_ras_fix<D, LM, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  return DCG_OK;
+}
+
+template <int D, int LM>
+void fx_launch(const Level& L, const FixArgs& a, bool z_zero, cudaStream_t s) {
+  const size_t smem = fx_smem<D, LM>(L);
+  constexpr int nt = fx_threads(D, LM);
+  if (z_zero)
+    k_ras_fix<D, LM, true><<<L.nwork, nt, smem, s>>>(a, (const double*)L.f, (const double*)L.z, (double*)L.y);
+  else
+    k_ras_fix<D, LM, false><<<L.nwork, nt, smem, s>>>(a, (const double*)L.f, (const double*)L.z, (double*)L.y);
+}
+
+// compile-time extent that serves a level's largest box extent
+int fx_lm(int dim, int lmax) {
+  if (dim == 3) return lmax <= 4 ? 4 : 6;
+  return lmax <= 4 ? 4 : lmax <= 6 ? 6 : lmax <= 8 ? 8 : lmax <= 10 ? 10 : lmax <= 12 ? 12 : 16;
+}
+
+}  // namespace
+
+int ras_fix_batch(int dim, int lmax) { return fx_batch(dim, fx_lm(dim, lmax)); }
+
+// Tables of a level's box classes and its quantisation (see the file header).
+int ras_fix_setup(dcg_problem* p, Level& L, cudaStream_t s) {
+  typedef long double ld;
+  const int D = p->dim, LM = fx_lm(D, L.fdm_lmax), HM = (LM + 1) / 2, HP = fx_hm(LM);
+  const ld pi = acosl(-1.0L);
+  // A' = A / hs = rho * (the operator at h = 1)
+  ld rho = 1.0L;
+  L.fx_sf = 0;
+  if (D == 3) {
+    int e = 0;
+    const ld fr = frexpl(1.0L / L.n, &e);  // h = fr 2^e, fr in [0.5, 1)
+    rho = 2.0L * fr;
+    L.fx_sf = -(e - 1);
+  }
+  // Constants are formed in extended precision, once per extent and per pair
+  // of extents along y and z (extended precision is software on Arm), and
+  // kept as integers C = round(c 2^58); the bounds need doubles only.
+  struct Ext {
+    std::vector<ld> kap, mu;    // 1D eigenvalues at h = 1
+    std::vector<long long> S;   // sine matrix
+    double row = 0.0, mx = 0.0; // largest absolute row sum and entry of S
+  };
+  std::map<int, Ext> ext;
+  int nmax = 0;
+  for (const auto& c : L.classes) {
+    nmax = std::max(nmax, c.len[0]);
+    for (int k = 0; k < D; ++k) {
+      const int l = c.len[k];
+      if (ext.count(l)) continue;
+      Ext& e = ext[l];
+      const ld nrm = sqrtl(2.0L / (l + 1));
+      std::vector<long long> sn(l + 1);
+      for (int j = 0; j <= l; ++j) sn[j] = j == 0 ? 0 : fx_const_bits(nrm * sinl(pi * j / (l + 1)));
+      for (int j = 0; j < l; ++j) {
+        double t = 0.0;
+        for (int x = 0; x < l; ++x) {
+          const int a = ((j + 1) * (x + 1)) % (2 * (l + 1));
+          e.S.push_back(a <= l ? sn[a] : a == l + 1 ? 0 : -sn[a - l - 1]);
+          const double v = std::fabs(std::ldexp((double)e.S.back(), -58));
+          t += v;
+          e.mx = std::max(e.mx, v);
+        }
+        e.row = std::max(e.row, t);
+        const ld cs = cosl(pi * (j + 1) / (l + 1));
+        e.kap.push_back(2.0L * (1.0L - cs));
+        e.mu.push_back((2.0L + cs) / 3.0L);
+      }
+    }
+  }
+  // Line systems along x after the transforms along y (j) and z (k): the
+  // tridiagonal Toeplitz part of A', the same for every extent along x (a
+  // shorter line takes the first factors). Per row i: -l_i, winv_i,
+  // -b winv_i, and the reciprocal pivot of the row that meets an equal
+  // elimination of i + 1 rows from the other end.
+  struct Line {
+    std::vector<long long> l, w, bw, meet;
+    std::vector<double> ld_, wd;  // |l_i| and winv_i
+    double b;
+  };
+  std::map<std::pair<int, int>, std::vector<Line>> lines;
+  for (const auto& c : L.classes) {
+    const std::pair<int, int> key(c.len[1], D == 2 ? 1 : c.len[2]);
+    if (lines.count(key)) continue;
+    std::vector<Line>& v = lines[key];
+    const Ext &ey = ext[c.len[1]], &ez = ext[c.len[D - 1]];
+    for (int sys = 0; sys < key.first * key.second; ++sys) {
+      const int j = sys % key.first, k = sys / key.first;
+      const ld cm = D == 2 ? ey.kap[j] / 2.0L : (ey.kap[j] * ez.mu[k] + ey.mu[j] * ez.kap[k]) / 3.0L;
+      const ld ck = D == 2 ? ey.mu[j] / 2.0L : ey.mu[j] * ez.mu[k] / 3.0L;
+      const ld a = rho * (cm * (4.0L / 6.0L) + ck * 2.0L), bb = rho * (cm / 6.0L - ck);
+      Line r;
+      r.b = std::fabs((double)bb);
+      ld wi = 0.0L;  // reciprocal pivot
+      for (int i = 0; i < nmax; ++i) {
+        const ld li = bb * wi, w = a - li * bb;
+        wi = 1.0L / w;
+        const ld bw = bb * wi;
+        r.l.push_back(fx_const_bits(-li));
+        r.w.push_back(fx_const_bits(wi));
+        r.bw.push_back(fx_const_bits(-bw));
+        r.meet.push_back(fx_const_bits(1.0L / (w - bb * bw)));
+        r.ld_.push_back(std::fabs((double)li));
+        r.wd.push_back((double)wi);
+      }
+      v.push_back(r);
+    }
+  }
+  auto lines_of = [&](const RasClass& c) -> const std::vector<Line>& {
+    return lines.at(std::pair<int, int>(c.len[1], D == 2 ? 1 : c.len[2]));
+  };
+  // ||T^-1||_inf of a line of n rows: |T^-1| is the inverse with off-diagonals
+  // -|b|, and its row sums solve that system for a right-hand side of ones;
+  // *grow: bound of the forward sweep for |g| <= 1
+  auto line_norm = [&](const Line& r, int n, double* grow) {
+    std::vector<double> v(n);
+    double u = 0.0, norm = 0.0;
+    for (int i = 0; i < n; ++i) {
+      v[i] = u = 1.0 + r.ld_[i] * u;
+      *grow = std::max(*grow, u);
+    }
+    for (int i = n - 1; i >= 0; --i) {
+      v[i] = (v[i] + (i + 1 < n ? r.b * v[i + 1] : 0.0)) * r.wd[i];
+      norm = std::max(norm, v[i]);
+    }
+    return norm;
+  };
+  double t1 = 1.0, grow = 1.0, norm = 1.0;
+  std::vector<std::vector<double>> norms(L.classes.size());
+  for (size_t q = 0; q < L.classes.size(); ++q) {
+    const RasClass& c = L.classes[q];
+    for (const Line& r : lines_of(c)) {
+      norms[q].push_back(line_norm(r, c.len[0], &grow));
+      norm = std::max(norm, norms[q].back());
+    }
+    for (int ax = 1; ax < D; ++ax) t1 = std::max(t1, ext[c.len[ax]].row);
+  }
+  // Quantisation: every operand of a multiply-add stays 1% below 2^60.
+  // g bits of residual allow the fold (2), the transforms (t1 per axis), the
+  // forward elimination (grow) and, in units of 2^K, the line solutions
+  // (norm) and in 3D their transform back along y, which is also the
+  // transform along z of the box's solution (bounded by t1 norm_box; norm of
+  // the lines times t1^2 bounds both).
+  const double lim = 0.99 * std::ldexp(1.0, 60);
+  auto bits_below = [&](double factor) { return (int)std::floor(std::log2(lim / factor)); };
+  const double kappa = D == 2 ? 1.0 / 6.0 : (double)rho / 36.0;
+  const double tz = D == 2 ? 16.0 : 64.0;  // sum of the |coefficients| of T
+  const double tD = D == 2 ? t1 : t1 * t1;
+  double solve = std::max(2.0, tD * grow);
+  if (D == 3) solve = std::max(solve, 2.0 * t1);
+  L.fx_gb = bits_below(solve);
+  std::vector<std::vector<int>> K(L.classes.size());
+  L.fx_kout = 0;
+  int k3 = 0;  // 3D: one K for every line
+  if (D == 3) {
+    // trade bits of the residual for bits of the solution
+    const int g0 = L.fx_gb;
+    auto gb_of = [&](int k) { return std::min(g0, bits_below(t1 * tD * norm * std::ldexp(1.0, -k))); };
+    for (int k = 0; k < 16; ++k)
+      if (gb_of(k) - k > gb_of(k3) - k3 || gb_of(k3) < g0 - 1 || norm * std::ldexp(1.0, -k3) > 1.99) k3 = k;
+    L.fx_gb = gb_of(k3);
+    L.fx_kout = std::max(0, k3 - 1);
+  }
+  for (size_t q = 0; q < L.classes.size(); ++q) {
+    const Ext& ey = ext[L.classes[q].len[1]];
+    for (double nr : norms[q]) {
+      int k = k3;
+      if (D == 2) {
+        while (bits_below(t1 * nr * std::ldexp(1.0, -k)) < L.fx_gb || nr * std::ldexp(1.0, -k) > 1.99) ++k;
+        // units of the results such that S 2^(K_j - kout) < 2
+        while (ey.mx * std::ldexp(1.0, k - L.fx_kout) > 1.99) ++L.fx_kout;
+      }
+      K[q].push_back(k);
+    }
+  }
+  L.fx_zb = std::min(bits_below(tz), L.fx_gb - (int)std::ceil(std::log2(1.0 + kappa * tz)));
+  L.fx_kappa = fx_const(fx_const_bits(D == 2 ? 1.0L / 6.0L : rho / 36.0L));
+
+  std::vector<int2> tab;
+  for (size_t q = 0; q < L.classes.size(); ++q) {
+    RasClass& c = L.classes[q];
+    const int2 none = make_int2(0, 0);
+    for (int ax = 0; ax < D - 1; ++ax) {
+      const int l = c.len[ax + 1], hc = (l + 1) / 2;
+      const std::vector<long long>& S = ext[l].S;
+      c.fx_f[ax] = (int)tab.size();
+      for (int j = 0; j < LM; ++j)
+        for (int x = 0; x < HP; ++x)
+          tab.push_back(j < l && x < hc && !((j & 1) && 2 * x + 1 == l) ? fx_const(S[j * l + x]) : none);
+      c.fx_b[ax] = (int)tab.size();
+      for (int x = 0; x < HM; ++x)
+        for (int par = 0; par < 2; ++par)
+          for (int k = 0; k < HP; ++k) {
+            const int j = 2 * k + par;
+            const bool in = j < l && x < hc && !(par && 2 * x + 1 == l);
+            // the last transform back (2D: y, 3D: z) goes to the units of the results
+            const int sc = !in ? 0 : D == 2 ? K[q][j] - L.fx_kout : ax == 1 ? k3 - L.fx_kout : 0;
+            tab.push_back(in ? fx_const(S[j * l + x], sc) : none);
+          }
+    }
+    c.fx_tri = (int)tab.size();
+    const std::vector<Line>& ln = lines_of(c);
+    const int n = c.len[0], nsys = (int)ln.size();
+    for (int sys = 0; sys < nsys; ++sys)
+      if (!(norms[q][sys] * std::ldexp(1.0, -K[q][sys]) < 2.0)) {
+        set_error_msg("fixed-point smoother: line factor out of range");
+        return DCG_ERR_UNSUPPORTED;
+      }
+    for (int i = 0; i < n; ++i)
+      for (int sys = 0; sys < nsys; ++sys) tab.push_back(fx_const(ln[sys].l[i]));
+    for (int i = 0; i < n; ++i)
+      for (int sys = 0; sys < nsys; ++sys) tab.push_back(fx_const(ln[sys].w[i], -K[q][sys]));
+    for (int i = 0; i < n; ++i)
+      for (int sys = 0; sys < nsys; ++sys) tab.push_back(fx_const(ln[sys].bw[i]));
+    for (int sys = 0; sys < nsys; ++sys)
+      tab.push_back(n % 2 == 0 ? fx_const(ln[sys].meet[n / 2 - 1], -K[q][sys]) : none);
+  }
+  DCG_CUDA(cudaMalloc(&L.d_fix, sizeof(int2) * tab.size()));
+  DCG_CUDA(cudaMemcpyAsync(L.d_fix, tab.data(), sizeof(int2) * tab.size(), cudaMemcpyHostToDevice, s));
+  DCG_CUDA(cudaStreamSynchronize(s));  // the host table goes out of scope
+  if (D == 3) return LM == 4 ? fx_attr<3, 4>(L) : fx_attr<3, 6>(L);
+  switch (LM) {
+    case 4: return fx_attr<2, 4>(L);
+    case 6: return fx_attr<2, 6>(L);
+    case 8: return fx_attr<2, 8>(L);
+    case 10: return fx_attr<2, 10>(L);
+    case 12: return fx_attr<2, 12>(L);
+    default: return fx_attr<2, 16>(L);
+  }
+}
+
+// y = exact local solves of r = f - Z z on every box (z_zero: of f)
+int ras_fix_solve(dcg_problem* p, const Level& L, bool z_zero, cudaStream_t s) {
+  FixArgs a{};
+  a.work = L.d_work;
+  a.class_patches = L.d_class_patches;
+  a.classes = L.d_classes;
+  a.origin = L.d_origin;
+  a.item_off = L.d_item_off;
+  a.tab = L.d_fix;
+  a.m = L.m;
+  a.bits = z_zero ? L.fx_gb : L.fx_zb;
+  a.sf = L.fx_sf;
+  a.kout = L.fx_kout;
+  a.kappa = L.fx_kappa;
+  const int LM = fx_lm(p->dim, L.fdm_lmax);
+  if (p->dim == 3) {
+    if (LM == 4) fx_launch<3, 4>(L, a, z_zero, s);
+    else fx_launch<3, 6>(L, a, z_zero, s);
+  } else {
+    switch (LM) {
+      case 4: fx_launch<2, 4>(L, a, z_zero, s); break;
+      case 6: fx_launch<2, 6>(L, a, z_zero, s); break;
+      case 8: fx_launch<2, 8>(L, a, z_zero, s); break;
+      case 10: fx_launch<2, 10>(L, a, z_zero, s); break;
+      case 12: fx_launch<2, 12>(L, a, z_zero, s); break;
+      default: fx_launch<2, 16>(L, a, z_zero, s);
+    }
+  }
+  DCG_LAUNCH_CHECK();
+  return DCG_OK;
+}
+
+}  // namespace dcg
