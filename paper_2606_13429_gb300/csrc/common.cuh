@@ -386,12 +386,24 @@ int q_from_t(dcg_problem* p, const double* t, const double* zh, const double* dv
              cudaStream_t s);
 // divergence stencil G[p*3+q][offset] of the uniform Q1 mesh (d = 2, 3)
 void div_stencil(int d, int n, double (*gs)[27]);
-// matrix-free 3D product (mf.cu): operand mode xm (0 x, 1 x - V zh, 2 V zh),
-// output mode om (0 y, 1 f - y, 2 V^T y), fused dot when `dot`, FP32
-// arithmetic when `lowp`
-int mf_product(dcg_problem* p, int xm, int om, bool dot, bool lowp, const double* x, const double* zh,
-               const double* f, double* y, const double* dvec, Reduce red, cudaStream_t s);
-// FP32 matrix-free products inside the outer iterations (mixed precision)
+// FP64 product with A in factored form (op.cu): operand x, x - V zh (both) or
+// V zh (x null); output y, f - y (f), V^T y (vt), or y and g = V^T y (g);
+// slot >= 0: dot (dvec, y), or the sum of squares of f - y, V^T y or g
+struct OpCall {
+  const double* x = nullptr;
+  const double* zh = nullptr;
+  const double* f = nullptr;
+  double* y = nullptr;
+  double* g = nullptr;
+  const double* dvec = nullptr;
+  bool vt = false;
+  int slot = -1;
+};
+int op_product(dcg_problem* p, const OpCall& c, cudaStream_t s);
+// matrix-free 3D product in FP32 arithmetic (mf.cu): operand mode xm (0 x, 1 x - V zh, 2 V zh),
+// output mode om (0 y, 2 V^T y), fused dot when `dot`
+int mf_product(dcg_problem* p, int xm, int om, bool dot, const double* x, const double* zh, double* y,
+               const double* dvec, Reduce red, cudaStream_t s);
 // inner stencil of a matrix-free problem, and its check against the operator
 int mf_probe_stencil(dcg_problem* p, double* stencil, cudaStream_t s);
 int mf_check_stencil(dcg_problem* p, cudaStream_t s);

@@ -1,4 +1,4 @@
-// Matrix-free product with the 3D pseudo-stress operator
+// Matrix-free product with the 3D pseudo-stress operator in FP32 arithmetic
 //
 //   y = sum_e P_e^T [ (1/(nu_e dt)) M_e (x) D_3 + G_e ] P_e x
 //
@@ -20,29 +20,22 @@
 // Layout: a CTA owns a 32 x 8 column of nodes and marches along z, keeping
 // three z-planes of the operand (halo included, zero outside the interior
 // grid) in shared memory, one array per component; each thread produces one
-// node per plane. T is the arithmetic type (float for the FP32 variant, whose
-// input and output stay FP64 in memory; double for the FP64 one). The
-// operand, output and dot-product variants are those of the BSR product.
+// node per plane. Input and output stay FP64 in memory (the FP64 product is
+// op.cu's).
 #include "common.cuh"
 
 namespace dcg {
 namespace {
 
-// tile: 32 x MY nodes per CTA, MY = 8 for FP32 and 4 for FP64 (the three
-// halo planes then take 37 KB and 44 KB of shared memory)
-constexpr int kMX = 32, kPX = kMX + 2;
-template <typename T>
-__host__ __device__ constexpr int mf_my() {
-  return sizeof(T) == 8 ? 4 : 8;
-}
+// tile: 32 x 8 nodes per CTA (the three halo planes take 37 KB of shared memory)
+constexpr int kMX = 32, kMY = 8, kPX = kMX + 2;
 
-enum MfX { MX_X = 0, MX_X_MINUS_VZ = 1, MX_VZ = 2 };
-enum MfO { MO_Y = 0, MO_FMY = 1, MO_VT = 2 };
+enum MfX { MX_X = 0, MX_X_MINUS_VZ = 1 };
+enum MfO { MO_Y = 0, MO_VT = 2 };
 
 struct MfArgs {
   const double* x;
   const double* zh;
-  const double* f;
   double* y;
   const double* dvec;
   const double* inv_nu;  // per element (n^3), or null: inv_nu_const
@@ -51,37 +44,22 @@ struct MfArgs {
   int m, n;
   int tiles_x, tiles_y, zchunk;
   Reduce red;
-  double mc64[27];      // h^3 prod(1/3 | 1/6) / dt per offset
-  float mc32[27];
-  double gs64[9][27];   // divergence stencil [p*3+q][offset]
-  float gs32[9][27];
+  float mc[27];         // h^3 prod(1/3 | 1/6) / dt per offset
+  float gs[9][27];      // divergence stencil [p*3+q][offset]
 };
-
-template <typename T>
-__device__ __forceinline__ T mc_of(const MfArgs& A, int o);
-template <>
-__device__ __forceinline__ float mc_of<float>(const MfArgs& A, int o) { return A.mc32[o]; }
-template <>
-__device__ __forceinline__ double mc_of<double>(const MfArgs& A, int o) { return A.mc64[o]; }
-template <typename T>
-__device__ __forceinline__ T gs_of(const MfArgs& A, int pq, int o);
-template <>
-__device__ __forceinline__ float gs_of<float>(const MfArgs& A, int pq, int o) { return A.gs32[pq][o]; }
-template <>
-__device__ __forceinline__ double gs_of<double>(const MfArgs& A, int pq, int o) { return A.gs64[pq][o]; }
 
 template <int XM>
 __device__ __forceinline__ double operand(const MfArgs& A, long long a, int c) {
   const bool diag = (c & 3) == 0;  // components 0, 4, 8
   if (XM == MX_X) return __ldg(A.x + a * 9 + c);
-  if (XM == MX_VZ) return diag ? A.isd * __ldg(A.zh + a) : 0.0;
   const double v = __ldg(A.x + a * 9 + c);
   return diag ? v - A.isd * __ldg(A.zh + a) : v;
 }
 
-template <typename T, int XM, int OM, bool DOT>
-__global__ void __launch_bounds__(kMX * mf_my<T>()) k_mf(MfArgs A) {
-  constexpr int kMY = mf_my<T>(), kMT = kMX * kMY, kPY = kMY + 2;
+template <int XM, int OM, bool DOT>
+__global__ void __launch_bounds__(kMX * kMY) k_mf(MfArgs A) {
+  using T = float;
+  constexpr int kMT = kMX * kMY, kPY = kMY + 2;
   __shared__ T pl[3][9][kPY][kPX];
   const int tx = threadIdx.x & (kMX - 1), ty = threadIdx.x / kMX;
   const int m = A.m;
@@ -168,18 +146,18 @@ __global__ void __launch_bounds__(kMX * mf_my<T>()) k_mf(MfArgs A) {
             T xn[9];
 #pragma unroll
             for (int c = 0; c < 9; ++c) xn[c] = pl[slot][c][ty + oy][tx + ox];
-            const T cm = W[oz][oy][ox] * mc_of<T>(A, o);
+            const T cm = W[oz][oy][ox] * A.mc[o];
 #pragma unroll
             for (int c = 0; c < 9; ++c) ym[c] = fma(cm, xn[c], ym[c]);
 #pragma unroll
             for (int p = 0; p < 3; ++p) {
-              const T gpp = gs_of<T>(A, p * 3 + p, o);
+              const T gpp = A.gs[p * 3 + p][o];
 #pragma unroll
               for (int k = 0; k < 3; ++k) yg[k * 3 + p] = fma(gpp, xn[k * 3 + p], yg[k * 3 + p]);
 #pragma unroll
               for (int q = 0; q < 3; ++q) {
                 if (q == p || oc[p] == 1 || oc[q] == 1) continue;  // cross stencil is zero there
-                const T gpq = gs_of<T>(A, p * 3 + q, o);
+                const T gpq = A.gs[p * 3 + q][o];
 #pragma unroll
                 for (int k = 0; k < 3; ++k) yg[k * 3 + p] = fma(gpq, xn[k * 3 + q], yg[k * 3 + p]);
               }
@@ -200,10 +178,9 @@ __global__ void __launch_bounds__(kMX * mf_my<T>()) k_mf(MfArgs A) {
       } else {
 #pragma unroll
         for (int c = 0; c < 9; ++c) {
-          double v = out[c];
-          if (OM == MO_FMY) v = A.f[a * 9 + c] - v;
+          const double v = out[c];
           A.y[a * 9 + c] = v;
-          if (DOT) part[0] = (OM == MO_FMY) ? fma(v, v, part[0]) : fma(A.dvec[a * 9 + c], v, part[0]);
+          if (DOT) part[0] = fma(A.dvec[a * 9 + c], v, part[0]);
         }
       }
     }
@@ -219,12 +196,12 @@ void build_tables(MfArgs& a, int n, double dt) {
     const int off[3] = {o % 3 - 1, (o / 3) % 3 - 1, o / 9 - 1};
     double mc = 1.0 / dt;
     for (int ax = 0; ax < 3; ++ax) mc *= off[ax] == 0 ? h / 3.0 : h / 6.0;
-    a.mc64[o] = mc;
-    a.mc32[o] = (float)mc;
+    a.mc[o] = (float)mc;
   }
-  div_stencil(3, n, a.gs64);
+  double gs64[9][27];
+  div_stencil(3, n, gs64);
   for (int pq = 0; pq < 9; ++pq)
-    for (int o = 0; o < 27; ++o) a.gs32[pq][o] = (float)a.gs64[pq][o];
+    for (int o = 0; o < 27; ++o) a.gs[pq][o] = (float)gs64[pq][o];
 }
 
 __global__ void k_unit(double* v, long long i) { v[i] = 1.0; }
@@ -241,23 +218,23 @@ __global__ void k_sub_inplace(double* a, const double* b, long long n) {
     a[i] -= b[i];
 }
 
-template <typename T, int XM, int OM, bool DOT>
+template <int XM, int OM, bool DOT>
 void launch_mf(MfArgs a, cudaStream_t s) {
   // z chunks: enough CTAs for every SM to hold several (two halo planes per chunk)
   a.tiles_x = (a.m + kMX - 1) / kMX;
-  a.tiles_y = (a.m + mf_my<T>() - 1) / mf_my<T>();
+  a.tiles_y = (a.m + kMY - 1) / kMY;
   const long long cols = (long long)a.tiles_x * a.tiles_y;
   long long nzc = (4 * 152 + cols - 1) / cols;
   nzc = std::max(1LL, std::min(nzc, (long long)(a.m + 7) / 8));
   a.zchunk = (int)((a.m + nzc - 1) / nzc);
   nzc = (a.m + a.zchunk - 1) / a.zchunk;
-  k_mf<T, XM, OM, DOT><<<(unsigned)(cols * nzc), kMX * mf_my<T>(), 0, s>>>(a);
+  k_mf<XM, OM, DOT><<<(unsigned)(cols * nzc), kMX * kMY, 0, s>>>(a);
 }
 
 }  // namespace
 
-int mf_product(dcg_problem* p, int xm, int om, bool dot, bool lowp, const double* x, const double* zh,
-               const double* f, double* y, const double* dvec, Reduce red, cudaStream_t s) {
+int mf_product(dcg_problem* p, int xm, int om, bool dot, const double* x, const double* zh, double* y,
+               const double* dvec, Reduce red, cudaStream_t s) {
   if (p->dim != 3) {
     set_error_msg("matrix-free product is implemented for 3D meshes");
     return DCG_ERR_UNSUPPORTED;
@@ -265,7 +242,6 @@ int mf_product(dcg_problem* p, int xm, int om, bool dot, bool lowp, const double
   MfArgs a;
   a.x = x;
   a.zh = zh;
-  a.f = f;
   a.y = y;
   a.dvec = dvec;
   a.inv_nu = p->inv_nu_elem;
@@ -284,36 +260,34 @@ int mf_product(dcg_problem* p, int xm, int om, bool dot, bool lowp, const double
   }
   // algorithmic work per node: 27 x 9 mass FMAs, 27 x 9 diagonal and
   // 6 x 12 x 3 cross divergence FMAs; bytes: operand, 1/nu (one element per
-  // node), output, and f or dvec when read
+  // node), output, and dvec when read
   const double nn = (double)p->n_nodes;
   const double flops = 2.0 * (243 + 243 + 216) * nn;
-  double bytes = (xm == MX_VZ ? 8.0 : 72.0) * nn + (xm == MX_X_MINUS_VZ ? 8.0 : 0.0) * nn;
+  double bytes = 72.0 * nn + (xm == MX_X_MINUS_VZ ? 8.0 : 0.0) * nn;
   bytes += (p->inv_nu_elem ? 8.0 : 0.0) * nn + (om == MO_VT ? 8.0 : 72.0) * nn;
-  if (om == MO_FMY || (dot && om == MO_Y)) bytes += 72.0 * nn;
+  if (dot && om == MO_Y) bytes += 72.0 * nn;
   const int prof = prof_begin(p, PC_SPMV, s);
-#define DCG_MF(T, XMV, OMV, DT) launch_mf<T, XMV, OMV, DT>(a, s)
-#define DCG_MF_T(XMV, OMV, DT) \
-  do {                          \
-    if (lowp) DCG_MF(float, XMV, OMV, DT); \
-    else DCG_MF(double, XMV, OMV, DT);     \
-  } while (0)
-  if (xm == MX_X && om == MO_Y && !dot) DCG_MF_T(MX_X, MO_Y, false);
-  else if (xm == MX_X && om == MO_Y && dot) DCG_MF_T(MX_X, MO_Y, true);
-  else if (xm == MX_X && om == MO_FMY) DCG_MF_T(MX_X, MO_FMY, true);
-  else if (xm == MX_X && om == MO_VT) DCG_MF_T(MX_X, MO_VT, true);
-  else if (xm == MX_VZ && om == MO_Y) DCG_MF_T(MX_VZ, MO_Y, false);
-  else if (xm == MX_VZ && om == MO_FMY) DCG_MF_T(MX_VZ, MO_FMY, true);
-  else if (xm == MX_VZ && om == MO_VT) DCG_MF_T(MX_VZ, MO_VT, true);
-  else if (xm == MX_X_MINUS_VZ && om == MO_Y) DCG_MF_T(MX_X_MINUS_VZ, MO_Y, true);
+  if (xm == MX_X && om == MO_Y && !dot) launch_mf<MX_X, MO_Y, false>(a, s);
+  else if (xm == MX_X && om == MO_Y) launch_mf<MX_X, MO_Y, true>(a, s);
+  else if (xm == MX_X && om == MO_VT && dot) launch_mf<MX_X, MO_VT, true>(a, s);
+  else if (xm == MX_X_MINUS_VZ && om == MO_Y && dot) launch_mf<MX_X_MINUS_VZ, MO_Y, true>(a, s);
   else {
     set_error_msg("matrix-free product: unsupported operand/output combination");
     return DCG_ERR_UNSUPPORTED;
   }
-#undef DCG_MF_T
-#undef DCG_MF
   DCG_LAUNCH_CHECK();
   prof_end(p, prof, s, flops, bytes);
   return DCG_OK;
+}
+
+// g = V^T A V e (FP64)
+static int vz_vt(dcg_problem* p, const double* e, double* g, cudaStream_t s) {
+  OpCall c;
+  c.zh = e;
+  c.y = g;
+  c.vt = true;
+  c.slot = S_TMP0;
+  return op_product(p, c, s);
 }
 
 // Z_J = V^T A V read off the operator: the column of a unit vector at an
@@ -332,7 +306,7 @@ int mf_probe_stencil(dcg_problem* p, double* stencil, cudaStream_t s) {
   if (cudaMemsetAsync(e, 0, sizeof(double) * nn, s) != cudaSuccess) st = DCG_ERR_CUDA;
   if (st == DCG_OK) {
     k_unit<<<1, 1, 0, s>>>(e, c);
-    st = mf_product(p, MX_VZ, MO_VT, true, false, nullptr, e, nullptr, g, nullptr, make_reduce(p, S_TMP0), s);
+    st = vz_vt(p, e, g, s);
   }
   for (int o = 0; o < 27 && st == DCG_OK; ++o) {
     const long long nb = c + (o % 3 - 1) + m * ((o / 3) % 3 - 1) + m * m * (o / 9 - 1);
@@ -360,7 +334,7 @@ int mf_check_stencil(dcg_problem* p, cudaStream_t s) {
   }
   const int g = grid_for(nn, 256, 4096);
   k_pattern_vec<<<g, 256, 0, s>>>(z, nn);
-  int st = mf_product(p, MX_VZ, MO_VT, true, false, nullptr, z, nullptr, y1, nullptr, make_reduce(p, S_TMP0), s);
+  int st = vz_vt(p, z, y1, s);
   if (st == DCG_OK) st = mg_inner_apply(p, z, y2, s);
   if (st == DCG_OK) {
     k_sub_inplace<<<g, 256, 0, s>>>(y1, y2, nn);

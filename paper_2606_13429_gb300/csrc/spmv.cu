@@ -1,5 +1,24 @@
+// Operator products of the solvers: FP64 products through the factored form
+// of op.cu (matrix-free problems and all but small assembled ones) or the
+// stored blocks (small assembled grids), FP32 matrix-free products through
+// mf.cu, and q = t - A V zh of the deflated product.
+//
+// Variants (x operand / output):
+//   x            : y = A x
+//   x - V zh     : q = A (d - V zh)          (M_D of Algorithm 2, second product)
+//   V zh         : y = A V zh                 (A pi(f) for f_D)
+//   out = y / f - y / V^T y / y and V^T y.
+#include "common.cuh"
+
+#include <cmath>
+
+namespace dcg {
+namespace {
+
 // FP64 BSR SpMV for the pseudo-stress operator, with the deflation
-// embed/extract and the CG dot products fused into its prologue/epilogue.
+// embed/extract and the CG dot products fused into its prologue/epilogue: the
+// product of small assembled grids (bsr_better below), where its short
+// independent sums beat the factored product of op.cu.
 //
 // Mapping in 2D (4 x 4 blocks): a CTA owns 32 consecutive block rows; warp w
 // computes scalar row R(w) of each of them (lane = block row). Every warp
@@ -16,11 +35,6 @@
 //   V zh         : y = A V zh                 (A pi(f) for f_D)
 //   out = y / f - y / V^T y (only the d diagonal-component rows are computed:
 //   g = V^T A x reads half (2D) or a third (3D) of the matrix).
-#include "common.cuh"
-
-namespace dcg {
-namespace {
-
 enum XMode { XM_X = 0, XM_X_MINUS_VZ = 1, XM_VZ = 2 };
 enum OMode { OM_Y = 0, OM_FMY = 1, OM_VT = 2, OM_YVT = 3 };
 
@@ -254,25 +268,8 @@ __global__ void __launch_bounds__(256) k_spmv3(SpmvArgs A) {
   if (DOT) grid_reduce<1>(part, A.red);
 }
 
-// w = x - V zh (node-major, the d diagonal components of each node shifted):
-// formed once per node instead of once per stored block that reads it, which
-// keeps the FP64 arithmetic of the deflated product at that of A x
-template <int D>
-__global__ void k_x_minus_vz(const double* __restrict__ x, const double* __restrict__ zh, double* __restrict__ w,
-                             long long nn, double isd) {
-  constexpr int B = D * D;
-  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < nn * B;
-       t += (long long)gridDim.x * blockDim.x) {
-    const long long a = t / B;
-    const int c = (int)(t - a * B);
-    const double v = x[t];
-    w[t] = (c % (D + 1) == 0) ? __dsub_rn(v, __dmul_rn(isd, __ldg(zh + a))) : v;
-  }
-}
-
 template <int XM, int OM, bool DOT>
-int launch(dcg_problem* p, SpmvArgs a, cudaStream_t s, bool lowp = false) {
-  if (p->matrix_free) return mf_product(p, XM, OM, DOT, lowp, a.x, a.zh, a.f, a.y, a.dvec, a.red, s);
+int launch(dcg_problem* p, SpmvArgs a, cudaStream_t s) {
   a.row_ptr = p->row_ptr;
   a.col_idx = p->col_idx;
   a.vals = p->vals;
@@ -303,86 +300,108 @@ int launch(dcg_problem* p, SpmvArgs a, cudaStream_t s, bool lowp = false) {
   return DCG_OK;
 }
 
+
+// The factored product walks a chain of rows or planes per thread, each FP64
+// instruction of a warp taking 64 clocks of its scheduler; on a small grid
+// that chain is the time, and the stored blocks (in L2 there) are faster.
+// Measured, uniform viscosity / one per element (us): 2D 95^2 6.8 / 8.2
+// against 5.0, 179^2 11.8 / 15.3 against 10.5, 256^2 11.8 / 15.4 against 18.6;
+// 3D 15^3 13.6 / 20.5 against 10.1, 19^3 13.7 / 20.6 against 19.3, 23^3 16.7 /
+// 25.3 against 39.5.
+// The 2D kernel reads x as 16-byte pairs: an operand that is only 8-byte
+// aligned goes to the factored product, which checks.
+bool bsr_better(const dcg_problem* p, const OpCall& c) {
+  return !p->matrix_free && p->n_nodes <= (p->dim == 2 ? 40000 : 8000) && (p->dim == 3 || !c.x || aligned16(c.x));
+}
+
+int bsr_product(dcg_problem* p, const OpCall& c, cudaStream_t s) {
+  SpmvArgs a{};
+  a.x = c.x;
+  a.zh = c.zh;
+  a.f = c.f;
+  a.y = c.y;
+  a.g = c.g;
+  a.dvec = c.dvec;
+  if (c.slot >= 0) a.red = make_reduce(p, c.slot);
+  if (!c.x) return c.f ? launch<XM_VZ, OM_FMY, true>(p, a, s) : launch<XM_VZ, OM_Y, false>(p, a, s);
+  if (c.zh) return launch<XM_X_MINUS_VZ, OM_Y, true>(p, a, s);
+  if (c.vt) return launch<XM_X, OM_VT, true>(p, a, s);
+  if (c.f) return launch<XM_X, OM_FMY, true>(p, a, s);
+  if (!c.g) return c.slot >= 0 ? launch<XM_X, OM_Y, true>(p, a, s) : launch<XM_X, OM_Y, false>(p, a, s);
+  if (p->dim == 3) return launch<XM_X, OM_YVT, true>(p, a, s);
+  // 2D: the plain product and the extraction g = V^T t as a separate pass,
+  // cheaper than the in-kernel exchange between the warps of the
+  // diagonal-component rows
+  DCG_TRY((launch<XM_X, OM_Y, false>(p, a, s)));
+  const int prof = prof_begin(p, PC_VEC, s);
+  DCG_TRY(vec_extract(p, c.y, c.g, c.slot, s));
+  prof_end(p, prof, s, 2.0 * p->n_nodes * p->dim, 8.0 * (2.0 * p->n_nodes + p->n_nodes));
+  return DCG_OK;
+}
+
+int product(dcg_problem* p, const OpCall& c, cudaStream_t s) {
+  return bsr_better(p, c) ? bsr_product(p, c, s) : op_product(p, c, s);
+}
+
 }  // namespace
 
 int spmv_plain(dcg_problem* p, const double* x, double* y, cudaStream_t s, bool lowp) {
-  SpmvArgs a{};
-  a.x = x;
-  a.y = y;
-  return launch<XM_X, OM_Y, false>(p, a, s, lowp);
+  if (lowp && p->matrix_free) return mf_product(p, 0, 0, false, x, nullptr, y, nullptr, Reduce{}, s);
+  OpCall c;
+  c.x = x;
+  c.y = y;
+  return product(p, c, s);
 }
 
 int spmv_dot(dcg_problem* p, const double* x, double* y, const double* dv, int slot, cudaStream_t s) {
-  SpmvArgs a{};
-  a.x = x;
-  a.y = y;
-  a.dvec = dv;
-  a.red = make_reduce(p, slot);
-  if (!dv) return launch<XM_X, OM_Y, false>(p, a, s);
-  return launch<XM_X, OM_Y, true>(p, a, s);
+  OpCall c;
+  c.x = x;
+  c.y = y;
+  c.dvec = dv;
+  if (dv) c.slot = slot;
+  return product(p, c, s);
 }
 
 int spmv_residual(dcg_problem* p, const double* f, const double* x, double* y, int slot, cudaStream_t s) {
-  SpmvArgs a{};
-  a.x = x;
-  a.f = f;
-  a.y = y;
-  a.red = make_reduce(p, slot);
-  return launch<XM_X, OM_FMY, true>(p, a, s);
+  OpCall c;
+  c.x = x;
+  c.f = f;
+  c.y = y;
+  c.slot = slot;
+  return product(p, c, s);
 }
 
 int spmv_vt(dcg_problem* p, const double* x, double* g, int slot, cudaStream_t s, bool lowp) {
-  SpmvArgs a{};
-  a.x = x;
-  a.y = g;
-  a.red = make_reduce(p, slot);
-  return launch<XM_X, OM_VT, true>(p, a, s, lowp);
+  if (lowp && p->matrix_free) return mf_product(p, 0, 2, true, x, nullptr, g, nullptr, make_reduce(p, slot), s);
+  OpCall c;
+  c.x = x;
+  c.y = g;
+  c.vt = true;
+  c.slot = slot;
+  return product(p, c, s);
 }
 
 int spmv_defl(dcg_problem* p, const double* x, const double* zh, double* q, int slot, cudaStream_t s, bool lowp) {
-  SpmvArgs a{};
-  a.x = x;
-  a.zh = zh;
-  a.y = q;
-  a.dvec = x;
-  a.red = make_reduce(p, slot);
-  if (!x) return launch<XM_VZ, OM_Y, false>(p, a, s, lowp);
-  if (!zh) return launch<XM_X, OM_Y, true>(p, a, s, lowp);
-  if (!p->matrix_free && p->sb.w) {
-    const double isd = 1.0 / std::sqrt((double)p->dim);
-    const int g = grid_for(p->N, 256, 8192);
-    const int prof = prof_begin(p, PC_VEC, s);
-    if (p->dim == 2) k_x_minus_vz<2><<<g, 256, 0, s>>>(x, zh, p->sb.w, p->n_nodes, isd);
-    else k_x_minus_vz<3><<<g, 256, 0, s>>>(x, zh, p->sb.w, p->n_nodes, isd);
-    DCG_LAUNCH_CHECK();
-    prof_end(p, prof, s, 2.0 * p->n_nodes * p->dim, 8.0 * (2.0 * p->N + p->n_nodes));
-    a.x = p->sb.w;  // dvec stays x: the fused dot is (x, A w)
-    return launch<XM_X, OM_Y, true>(p, a, s, lowp);
+  if (x && lowp && p->matrix_free)
+    return mf_product(p, zh ? 1 : 0, 0, true, x, zh, q, x, make_reduce(p, slot), s);
+  OpCall c;
+  c.x = x;
+  c.zh = zh;
+  c.y = q;
+  if (x) {
+    c.dvec = x;
+    c.slot = slot;
   }
-  return launch<XM_X_MINUS_VZ, OM_Y, true>(p, a, s, lowp);
+  return product(p, c, s);
 }
 
 int spmv_y_vt(dcg_problem* p, const double* x, double* t, double* g, int slot, cudaStream_t s) {
-  if (p->dim == 2) {
-    // 2D: the plain product (which streams the matrix at the rate of the
-    // lane-per-block-row layout) and the extraction g = V^T t as a separate
-    // pass over t: cheaper than the in-kernel exchange between the warps of
-    // the diagonal-component rows
-    SpmvArgs a{};
-    a.x = x;
-    a.y = t;
-    DCG_TRY((launch<XM_X, OM_Y, false>(p, a, s)));
-    const int prof = prof_begin(p, PC_VEC, s);
-    DCG_TRY(vec_extract(p, t, g, slot, s));
-    prof_end(p, prof, s, 2.0 * p->n_nodes * p->dim, 8.0 * (2.0 * p->n_nodes + p->n_nodes));
-    return DCG_OK;
-  }
-  SpmvArgs a{};
-  a.x = x;
-  a.y = t;
-  a.g = g;
-  a.red = make_reduce(p, slot);
-  return launch<XM_X, OM_YVT, true>(p, a, s);
+  OpCall c;
+  c.x = x;
+  c.y = t;
+  c.g = g;
+  c.slot = slot;
+  return product(p, c, s);
 }
 
 // Divergence part of the element blocks summed over elements: for the uniform
@@ -577,12 +596,12 @@ int q_from_t(dcg_problem* p, const double* t, const double* zh, const double* dv
 }
 
 int spmv_f_minus_avz(dcg_problem* p, const double* f, const double* zh, double* y, int slot, cudaStream_t s) {
-  SpmvArgs a{};
-  a.zh = zh;
-  a.f = f;
-  a.y = y;
-  a.red = make_reduce(p, slot);
-  return launch<XM_VZ, OM_FMY, true>(p, a, s);
+  OpCall c;
+  c.zh = zh;
+  c.f = f;
+  c.y = y;
+  c.slot = slot;
+  return product(p, c, s);
 }
 
 }  // namespace dcg
