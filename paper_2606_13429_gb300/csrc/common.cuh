@@ -217,6 +217,7 @@ struct Level {
   bool fdm = false;                 // FP64 local solves by fast diagonalisation and line solves
   int fdm_lmax = 0;                 // largest box extent along an axis (register bound of the kernel)
   int2* d_fix = nullptr;            // fixed-point sine matrices and line-solve factors of every class
+  int fx_ntab = 0;                  // its entries
   int fx_zb = 0, fx_gb = 0;         // bits of the quantised iterate and right-hand side / of a residual alone
   int fx_sf = 0, fx_kout = 0;       // exponent shifts of the right-hand side and of the results
   int2 fx_kappa{};                  // stencil factor
@@ -291,6 +292,7 @@ struct MGState {
   cudaGraphExec_t wexec = nullptr;
   bool fp32 = false;
   long long graph_kernels = 0;  // kernel launches captured into the W-cycle graph
+  void* small = nullptr;        // one-kernel solve of small hierarchies (small_mg.cu)
 };
 
 }  // namespace dcg
@@ -445,8 +447,16 @@ int mg_cycles(dcg_problem* p, const double* g, double* z, int ncycles, cudaStrea
 int mg_solve(dcg_problem* p, const double* g, double* z, double tol, int nmax, int* ncyc, cudaStream_t s);
 // FP64 smoother's local solves in 64-bit fixed point (ras_fix.cu)
 int ras_fix_batch(int dim, int lmax);
+int ras_fix_lm(int dim, int lmax);  // compile-time box extent that serves lmax
 int ras_fix_setup(dcg_problem* p, Level& L, cudaStream_t s);
 int ras_fix_solve(dcg_problem* p, const Level& L, bool z_zero, cudaStream_t s);
+// Algorithm 3 on small 2D FP64 hierarchies as one kernel (small_mg.cu)
+int small_mg_setup(dcg_problem* p, cudaStream_t s);
+void small_mg_free(dcg_problem* p);
+inline bool small_mg_ready(const dcg_problem* p) { return p->mg.small != nullptr && p->prof.mask == 0; }
+int small_mg_launch(dcg_problem* p, const double* g, double* z, double tol, int nmax, const double* tol_dev, int* total,
+                    int* iter, const int* in_iter, cudaStream_t s);
+int small_mg_cycles_done(dcg_problem* p, int* ncyc, cudaStream_t s);
 std::vector<int> level_sizes(int n, int max_levels);  // mesh sizes n_J, n_J/2, ... (finest first)
 int mg_ras_step_hook(dcg_problem* p, int level, const double* f, double* z, cudaStream_t s);
 // pieces of Algorithm 3 for the graph-captured solve (graph.cu)

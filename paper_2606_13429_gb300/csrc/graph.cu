@@ -262,6 +262,9 @@ struct Builder {
     k_g_inner_tol<<<1, 1, 0, s>>>(S, p->scal, in_iter);
     DCG_LAUNCH_CHECK();
     DCG_TRY(zero(z, p->n_nodes, s));
+    if (small_mg_ready(p))
+      return small_mg_launch(p, g, z, 0.0, p->opts.inner_nmax, &S->mg_tol, &S->total_cycles, &S->iter_cycles,
+                             &S->mg_in_iter, s);
     DCG_TRY(mg_graph_residual(p, g, z, true, s));
     cudaGraphConditionalHandle h = 0;
     DCG_TRY(handle(s, &h));

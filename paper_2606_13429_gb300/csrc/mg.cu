@@ -1595,7 +1595,9 @@ void free_level(Level& L) {
   L = Level{};
 }
 
-int setup_ras(dcg_problem* p, Level& L, bool fp32, cudaStream_t s) {
+// lmax_all: the largest box extent of any level (the levels share the
+// compile-time extent of their fixed-point tables)
+int setup_ras(dcg_problem* p, Level& L, bool fp32, int lmax_all, cudaStream_t s) {
   const int D = p->dim;
   const dcg_options& o = p->opts;
   L.tc = fp32 && o.ras_inverse == DCG_INV_BF16;  // BF16 inverses on the tensor cores
@@ -1639,8 +1641,8 @@ int setup_ras(dcg_problem* p, Level& L, bool fp32, cudaStream_t s) {
       dev = std::max(dev, std::fabs(cf.c[k] - L.st64.c[k]));
       mx = std::max(mx, std::fabs(cf.c[k]));
     }
-    L.fdm = dev <= 1e-12 * mx && lmax <= (D == 2 ? 16 : 6);
-    L.fdm_lmax = lmax;
+    L.fdm = dev <= 1e-12 * mx && lmax_all <= (D == 2 ? 16 : 6);
+    L.fdm_lmax = lmax_all;
   }
   L.ras_np2 = 0;
   for (int pid = 0; pid < L.npatch; ++pid) L.ras_np2 += (long long)L.classes[pclass[pid]].np * L.classes[pclass[pid]].np;
@@ -2064,6 +2066,7 @@ void mg_free(dcg_problem* p) {
   p->coarse = Coarse{};
   if (p->mg.wexec) cudaGraphExecDestroy(p->mg.wexec);
   if (p->mg.cap) cudaStreamDestroy(p->mg.cap);
+  small_mg_free(p);
   p->mg = MGState{};
 }
 
@@ -2208,12 +2211,14 @@ int mg_setup(dcg_problem* p, cudaStream_t s) {
   // --- buffers and RAS
   const size_t tsz = fp32 ? sizeof(float) : sizeof(double);
   p->mg.fp32 = fp32;
+  int lmax_all = 1;
+  for (int k = 1; k < J; ++k) lmax_all = std::max(lmax_all, std::min(p->levels[k].m, o.patch + 2 * o.overlap));
   for (int k = 0; k < J; ++k) {
     Level& L = p->levels[k];
     DCG_CUDA(cudaMalloc(&L.f, tsz * L.nn));
     DCG_CUDA(cudaMalloc(&L.z, tsz * L.nn));
     DCG_CUDA(cudaMemsetAsync(L.z, 0, tsz * L.nn, s));
-    if (k >= 1) DCG_TRY(setup_ras(p, L, fp32, s));
+    if (k >= 1) DCG_TRY(setup_ras(p, L, fp32, lmax_all, s));
   }
   // --- coarsest solver
   {
@@ -2300,7 +2305,10 @@ int mg_setup(dcg_problem* p, cudaStream_t s) {
   DCG_TRY(set_ras_smem(k_ras_solve<double, 3, false>));
   DCG_CUDA(cudaStreamSynchronize(s));
   if (p->matrix_free) DCG_TRY(mf_check_stencil(p, s));
-  if (!exact_mode(p)) DCG_TRY(build_wcycle_graph(p));
+  if (!exact_mode(p)) {
+    DCG_TRY(small_mg_setup(p, s));
+    DCG_TRY(build_wcycle_graph(p));
+  }
   return DCG_OK;
 }
 
@@ -2364,6 +2372,7 @@ int exact_solve(dcg_problem* p, const double* g, double* z, cudaStream_t s) {
 int mg_cycles(dcg_problem* p, const double* g, double* z, int ncycles, cudaStream_t s) {
   if (p->levels.empty()) return DCG_ERR_STATE;
   if (exact_mode(p)) return exact_solve(p, g, z, s);
+  if (small_mg_ready(p)) return small_mg_launch(p, g, z, -1.0, ncycles, nullptr, nullptr, nullptr, nullptr, s);
   const bool fp32 = p->mg.fp32;
   for (int c = 0; c < ncycles; ++c) {
     DCG_TRY(fp32 ? inner_residual<float>(p, g, z, s) : inner_residual<double>(p, g, z, s));
@@ -2382,6 +2391,10 @@ int mg_solve(dcg_problem* p, const double* g, double* z, double tol, int nmax, i
   if (p->levels.empty()) return DCG_ERR_STATE;
   *ncyc = 0;
   if (exact_mode(p)) return exact_solve(p, g, z, s);
+  if (small_mg_ready(p)) {
+    DCG_TRY(small_mg_launch(p, g, z, tol, nmax, nullptr, nullptr, nullptr, nullptr, s));
+    return small_mg_cycles_done(p, ncyc, s);
+  }
   const bool fp32 = p->mg.fp32;
   int n = 0;
   double gn = 0.0;

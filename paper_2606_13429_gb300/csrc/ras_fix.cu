@@ -51,7 +51,7 @@
 // lines of a class are padded by zero table entries up to the compile-time
 // LM. Results go to y box-major (y[item][b][i]).
 #include "common.cuh"
-#include "fix64.cuh"
+#include "ras_fix.cuh"
 
 #include <algorithm>
 #include <cmath>
@@ -68,163 +68,9 @@ struct FixArgs {
   const int4* origin;        // [npatch] box origin (x, y, z) and its node index
   const long long* item_off; // [nwork]
   const int2* tab;
-  int m, bits, sf, kout;     // bits: zb or gb; f is scaled by 2^sf
-  int2 kappa;                // r = f 2^sf + kappa T(z), T the integer stencil sum
+  int m;
+  FxScale sc;
 };
-
-constexpr int fx_group(int LM) { return LM + 2 <= 8 ? 8 : LM + 2 <= 16 ? 16 : 32; }  // lanes per box, 2D
-constexpr int fx_batch(int D, int LM) { return D == 2 ? 128 / fx_group(LM) : 8; }
-constexpr int fx_threads(int D, int LM) { return D == 2 ? 128 : 8 * LM * LM; }
-// CTAs per SM the register allocation leaves room for
-constexpr int fx_blocks(int D, int LM) { return D == 2 ? (LM <= 8 ? 7 : LM <= 12 ? 6 : 4) : (LM <= 4 ? 6 : 2); }
-// pitch of a line of table constants (pairs are read as 16-byte loads)
-__host__ __device__ constexpr int fx_hm(int LM) { return ((LM + 1) / 2 + 1) / 2 * 2; }
-
-// forward transform of one line in place; C[j][x], x < fx_hm(LM)
-template <int LM>
-__device__ __forceinline__ void fx_forward(long long* __restrict__ W, int stride, int l, const int2* __restrict__ C) {
-  constexpr int HM = (LM + 1) / 2, HP = fx_hm(LM);
-  const int h = l >> 1, hc = (l + 1) >> 1;
-  FxVal p[HP], q[HP];
-#pragma unroll
-  for (int x = 0; x < HP; ++x) {
-    const long long a = (x < HM && x < hc) ? W[x * stride] : 0;
-    const long long b = (x < HM && x < h) ? W[(l - 1 - x) * stride] : 0;
-    p[x] = fx_split(a + b);
-    q[x] = fx_split(a - b);
-  }
-  // two outputs per turn of a rolled loop: unrolled, the table loads of many
-  // outputs are hoisted together and take 250 registers
-#pragma unroll 1
-  for (int j = 0; j < l; j += 2) {
-    FxAcc e = fx_zero(), o = fx_zero();
-#pragma unroll
-    for (int x = 0; x < HP; x += 2) {
-      const int4 ce = *reinterpret_cast<const int4*>(C + j * HP + x);
-      const int4 co = *reinterpret_cast<const int4*>(C + (j + 1) * HP + x);
-      fx_mac(e, p[x], ce.x, ce.y);
-      fx_mac(o, q[x], co.x, co.y);
-      if (x + 1 < HM) {
-        fx_mac(e, p[x + 1], ce.z, ce.w);
-        fx_mac(o, q[x + 1], co.z, co.w);
-      }
-    }
-    W[j * stride] = fx_value(e);
-    if (j + 1 < l) W[(j + 1) * stride] = fx_value(o);
-  }
-}
-
-// transform back: out_x = sum_j C_x[j] v_j; C[x][j], x < (LM+1)/2, j < LM
-// (even j, then odd j, each padded to fx_hm(LM))
-template <int LM>
-__device__ __forceinline__ void fx_back(long long* __restrict__ W, int stride, int l, const int2* __restrict__ C) {
-  constexpr int HM = (LM + 1) / 2, HP = fx_hm(LM);
-  const int h = l >> 1, hc = (l + 1) >> 1;
-  FxVal v[2 * HP];
-#pragma unroll
-  for (int j = 0; j < 2 * HP; ++j) v[j] = fx_split((j < LM && j < l) ? W[j * stride] : 0);
-#pragma unroll 1
-  for (int x = 0; x < hc; ++x) {
-    FxAcc e = fx_zero(), o = fx_zero();
-#pragma unroll
-    for (int k = 0; k < HP; k += 2) {
-      const int4 ce = *reinterpret_cast<const int4*>(C + (2 * x) * HP + k);
-      const int4 co = *reinterpret_cast<const int4*>(C + (2 * x + 1) * HP + k);
-      fx_mac(e, v[2 * k], ce.x, ce.y);
-      fx_mac(o, v[2 * k + 1], co.x, co.y);
-      if (k + 1 < HM) {
-        fx_mac(e, v[2 * k + 2], ce.z, ce.w);
-        fx_mac(o, v[2 * k + 3], co.z, co.w);
-      }
-    }
-    const long long E = fx_value(e), O = fx_value(o);
-    W[x * stride] = E + O;
-    if (x < h) W[(l - 1 - x) * stride] = E - O;
-  }
-}
-
-// line solve in place. t: [4][n][nl] constants of this line with pitch nl:
-// -l_i; winv_i 2^-K; -b winv_i; and, for the exact extent n = LM, in entry
-// [3][0] the reciprocal pivot of the meeting row.
-// General extents: y_i = g_i - l_i y_{i-1}; x_i = winv_i y_i - b winv_i x_{i+1}.
-// n = LM: the line is Toeplitz, so it is eliminated from both ends with the
-// same factors, the two chains meeting at rows LM/2 - 1 and LM/2 (half the
-// dependent steps).
-template <int LM, bool EX>
-__device__ __forceinline__ void fx_line_solve(long long* __restrict__ W, int n, const int2* __restrict__ t, int nl) {
-  long long g[LM];
-#pragma unroll
-  for (int i = 0; i < LM; ++i) g[i] = (EX || i < n) ? W[i] : 0;
-  if constexpr (EX) {
-    constexpr int H = LM / 2;
-#pragma unroll
-    for (int i = 1; i < H; ++i) {
-      const int2 c = __ldg(t + i * nl);
-      FxAcc a = fx_zero(), d = fx_zero();
-      fx_mac(a, fx_split(g[i - 1]), c.x, c.y);
-      fx_mac(d, fx_split(g[LM - i]), c.x, c.y);
-      g[i] += fx_value(a);
-      g[LM - 1 - i] += fx_value(d);
-    }
-    // row H with the whole upper half eliminated
-    long long xa, xb;
-    {
-      const int2 c = __ldg(t + H * nl), cm = __ldg(t + 3 * LM * nl);
-      FxAcc a = fx_zero(), d = fx_zero();
-      fx_mac(a, fx_split(g[H - 1]), c.x, c.y);
-      fx_mac(d, fx_split(g[H] + fx_value(a)), cm.x, cm.y);
-      xb = fx_value(d);
-      W[H] = xb;
-    }
-    {
-      const int2 cw = __ldg(t + (LM + H - 1) * nl), cb = __ldg(t + (2 * LM + H - 1) * nl);
-      FxAcc a = fx_zero();
-      fx_mac(a, fx_split(g[H - 1]), cw.x, cw.y);
-      fx_mac(a, fx_split(xb), cb.x, cb.y);
-      xa = fx_value(a);
-      W[H - 1] = xa;
-    }
-#pragma unroll
-    for (int i = H - 2; i >= 0; --i) {
-      const int2 cw = __ldg(t + (LM + i) * nl), cb = __ldg(t + (2 * LM + i) * nl);
-      FxAcc a = fx_zero(), d = fx_zero();
-      fx_mac(a, fx_split(g[i]), cw.x, cw.y);
-      fx_mac(d, fx_split(g[LM - 1 - i]), cw.x, cw.y);
-      fx_mac(a, fx_split(xa), cb.x, cb.y);
-      fx_mac(d, fx_split(xb), cb.x, cb.y);
-      xa = fx_value(a);
-      xb = fx_value(d);
-      W[i] = xa;
-      W[LM - 1 - i] = xb;
-    }
-  } else {
-#pragma unroll
-    for (int i = 1; i < LM; ++i)
-      if (i < n) {
-        const int2 c = __ldg(t + i * nl);
-        FxAcc a = fx_zero();
-        fx_mac(a, fx_split(g[i - 1]), c.x, c.y);
-        g[i] += fx_value(a);
-      }
-    long long xn = 0;
-#pragma unroll
-    for (int i = LM - 1; i >= 0; --i)
-      if (i < n) {
-        const int2 cw = __ldg(t + (n + i) * nl), cb = __ldg(t + (2 * n + i) * nl);
-        FxAcc a = fx_zero();
-        fx_mac(a, fx_split(g[i]), cw.x, cw.y);
-        fx_mac(a, fx_split(xn), cb.x, cb.y);
-        xn = fx_value(a);
-        W[i] = xn;
-      }
-  }
-}
-
-// result of a box that is all zero, has a non-finite entry, or may overflow
-__device__ __forceinline__ double fx_special(long long v, int e0, unsigned mag) {
-  if (mag == 0) return 0.0;
-  return mag < kFxNonFinite ? fx_to_double(v, e0, false) : __longlong_as_double(0x7ff8000000000000ll);
-}
 
 // EX: the boxes have extent LM along every axis
 template <int LM, bool ZZERO, bool EX>
@@ -234,8 +80,6 @@ __device__ __forceinline__ void fx_boxes_2d(const FixArgs& A, const RasClass& C,
   constexpr int G = fx_group(LM), HP = fx_hm(LM), NF = LM * HP;
   const int lane = threadIdx.x & (G - 1), b = threadIdx.x / G;
   const int lx = EX ? LM : C.len[0], ly = EX ? LM : C.len[1], m = A.m;
-  const int wp = lx | 1;                     // row pitch of the box values
-  long long* W = smem + b * (ly * wp);       // [ly][wp]
   const bool live = b < cnt;                 // groups past the item's boxes only take part in the shuffles
   const int x = lane - 1;                    // column of the box, -1 and lx are its halo
   const bool own = live && x >= 0 && x < lx;
@@ -255,54 +99,9 @@ __device__ __forceinline__ void fx_boxes_2d(const FixArgs& A, const RasClass& C,
     for (int q = 0; q < LM; ++q)
       fv[q] = (own && q < ly) ? __double_as_longlong(__ldg(f + base + (q + 1) * m)) : 0;
   }
-  unsigned mag = 0;
-#pragma unroll
-  for (int q = 0; q < LM; ++q) mag = max(mag, fx_mag(fv[q]));
-  if (!ZZERO) {
-#pragma unroll
-    for (int q = 0; q < LM + 2; ++q) mag = max(mag, fx_mag(zv[q]));
-  }
-#pragma unroll
-  for (int o = G / 2; o > 0; o >>= 1) mag = max(mag, __shfl_xor_sync(0xffffffffu, mag, o, G));
-  const int e = fx_block_exponent(mag), sh0 = 63 - A.bits + e;
-  // residual r = f + kappa T(z), T = (sum of the 3 x 3 box) - 9 z
-  if (ZZERO) {
-#pragma unroll
-    for (int q = 0; q < LM; ++q)
-      if (own && q < ly) W[q * wp + x] = fx_near(fv[q], sh0);
-  } else {
-    long long s0 = 0, s1 = 0, zm = 0;
-#pragma unroll
-    for (int q = 0; q < LM + 2; ++q) {
-      const long long zc = fx_floor(zv[q], sh0);
-      const long long s2 = __shfl_up_sync(0xffffffffu, zc, 1, G) + zc + __shfl_down_sync(0xffffffffu, zc, 1, G);
-      if (q >= 2) {
-        const long long T = (s0 + s1 + s2) - (zm << 3) - zm;
-        FxAcc a = fx_zero();
-        fx_mac(a, fx_split(T), A.kappa.x, A.kappa.y);
-        if (own && q - 2 < ly) W[(q - 2) * wp + x] = fx_near(fv[q - 2], sh0) + fx_value(a);
-      }
-      s0 = s1;
-      s1 = s2;
-      zm = zc;
-    }
-  }
-  if (own) fx_forward<LM>(W + x, wp, ly, s_tab);
-  __syncwarp();
-  if (live && lane < ly) fx_line_solve<LM, EX>(W + lane * wp, lx, A.tab + C.fx_tri + lane, ly);
-  __syncwarp();
-  if (own) {
-    fx_back<LM>(W + x, wp, ly, s_tab + NF);
-    const int e0 = e + 63 - A.bits + A.kout;
-    const bool safe = mag != 0 && mag < kFxNonFinite && e0 < 0x7ff;
-    double* yb = yi + b * (lx * ly) + x;
-    if (safe) {
-#pragma unroll 4
-      for (int q = 0; q < ly; ++q) yb[q * lx] = fx_to_double(W[q * wp + x], e0, true);
-    } else {
-      for (int q = 0; q < ly; ++q) yb[q * lx] = fx_special(W[q * wp + x], e0, mag);
-    }
-  }
+  double* yb = yi + b * (lx * ly) + x;
+  fx_solve_2d<LM, ZZERO, EX>(A.sc, lx, ly, live, zv, fv, smem + b * (ly * (lx | 1)), s_tab, s_tab + NF,
+                             A.tab + C.fx_tri, [&](int q, double v) { yb[q * lx] = v; });
 }
 
 template <int LM, bool ZZERO, bool EX>
@@ -334,7 +133,7 @@ __device__ __forceinline__ void fx_boxes_3d(const FixArgs& A, const RasClass& C,
     for (int q = 0; q < LM; ++q) {
       fv[q] = (own && q < lz) ? __double_as_longlong(__ldg(f + base + (q + 1) * mm)) : 0;
       const unsigned mf = fx_mag(fv[q]);
-      mag = max(mag, mf >= kFxNonFinite || mf == 0 ? mf : (unsigned)max((int)mf + (A.sf << 20), 1));
+      mag = max(mag, mf >= kFxNonFinite || mf == 0 ? mf : (unsigned)max((int)mf + (A.sc.sf << 20), 1));
     }
     if (!ZZERO) {
 #pragma unroll
@@ -367,11 +166,11 @@ __device__ __forceinline__ void fx_boxes_3d(const FixArgs& A, const RasClass& C,
   if (live && mag) atomicMax(&s_e[b], mag);
   __syncthreads();
   mag = s_e[b];
-  const int e = fx_block_exponent(mag), sh0 = 63 - A.bits + e;
+  const int e = fx_block_exponent(mag), sh0 = 63 - A.sc.bits + e;
   if (ZZERO) {
 #pragma unroll
     for (int q = 0; q < LM; ++q)
-      if (own && q < lz) W[(q * ly + cy) * wp + cx] = fx_near(fv[q], sh0 - A.sf);
+      if (own && q < lz) W[(q * ly + cy) * wp + cx] = fx_near(fv[q], sh0 - A.sc.sf);
   } else {
 #pragma unroll
     for (int q = 0; q < LM + 2; ++q) {
@@ -394,8 +193,8 @@ __device__ __forceinline__ void fx_boxes_3d(const FixArgs& A, const RasClass& C,
         if (q >= 2) {
           const long long T = Em + Ep + (D0 << 1) - (zv[q - 1] << 5);
           FxAcc a = fx_zero();
-          fx_mac(a, fx_split(T), A.kappa.x, A.kappa.y);
-          if (q - 2 < lz) W[((q - 2) * ly + cy) * wp + cx] = fx_near(fv[q - 2], sh0 - A.sf) + fx_value(a);
+          fx_mac(a, fx_split(T), A.sc.kappa.x, A.sc.kappa.y);
+          if (q - 2 < lz) W[((q - 2) * ly + cy) * wp + cx] = fx_near(fv[q - 2], sh0 - A.sc.sf) + fx_value(a);
         }
         Em = E0;
         E0 = Ep;
@@ -417,7 +216,7 @@ __device__ __forceinline__ void fx_boxes_3d(const FixArgs& A, const RasClass& C,
   __syncthreads();
   if (own) {
     fx_back<LM>(W + cy * wp + cx, ly * wp, lz, s_tab + NF + NBK + NF);
-    const int e0 = e + 63 - A.bits + A.kout;
+    const int e0 = e + 63 - A.sc.bits + A.sc.kout;
     const bool safe = mag != 0 && mag < kFxNonFinite && e0 < 0x7ff;
     double* yb = yi + b * (lx * ly * lz) + cy * lx + cx;
     if (safe) {
@@ -502,6 +301,7 @@ int fx_lm(int dim, int lmax) {
 
 }  // namespace
 
+int ras_fix_lm(int dim, int lmax) { return fx_lm(dim, lmax); }
 int ras_fix_batch(int dim, int lmax) { return fx_batch(dim, fx_lm(dim, lmax)); }
 
 // Tables of a level's box classes and its quantisation (see the file header).
@@ -668,6 +468,7 @@ int ras_fix_setup(dcg_problem* p, Level& L, cudaStream_t s) {
     for (int ax = 0; ax < D - 1; ++ax) {
       const int l = c.len[ax + 1], hc = (l + 1) / 2;
       const std::vector<long long>& S = ext[l].S;
+      if (tab.size() & 1) tab.push_back(none);  // the transforms' tables are read as 16-byte pairs
       c.fx_f[ax] = (int)tab.size();
       for (int j = 0; j < LM; ++j)
         for (int x = 0; x < HP; ++x)
@@ -700,6 +501,7 @@ int ras_fix_setup(dcg_problem* p, Level& L, cudaStream_t s) {
     for (int sys = 0; sys < nsys; ++sys)
       tab.push_back(n % 2 == 0 ? fx_const(ln[sys].meet[n / 2 - 1], -K[q][sys]) : none);
   }
+  L.fx_ntab = (int)tab.size();
   DCG_CUDA(cudaMalloc(&L.d_fix, sizeof(int2) * tab.size()));
   DCG_CUDA(cudaMemcpyAsync(L.d_fix, tab.data(), sizeof(int2) * tab.size(), cudaMemcpyHostToDevice, s));
   DCG_CUDA(cudaStreamSynchronize(s));  // the host table goes out of scope
@@ -724,10 +526,7 @@ int ras_fix_solve(dcg_problem* p, const Level& L, bool z_zero, cudaStream_t s) {
   a.item_off = L.d_item_off;
   a.tab = L.d_fix;
   a.m = L.m;
-  a.bits = z_zero ? L.fx_gb : L.fx_zb;
-  a.sf = L.fx_sf;
-  a.kout = L.fx_kout;
-  a.kappa = L.fx_kappa;
+  a.sc = FxScale{z_zero ? L.fx_gb : L.fx_zb, L.fx_sf, L.fx_kout, L.fx_kappa};
   const int LM = fx_lm(p->dim, L.fdm_lmax);
   if (p->dim == 3) {
     if (LM == 4) fx_launch<3, 4>(L, a, z_zero, s);
