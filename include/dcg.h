@@ -327,8 +327,9 @@ int dcg_apply_div(const dcg_problem* p, const double* x, double* y, void* stream
  *   implicit Euler  b = (M_dev/alpha) s1 + F1
  *   Crank-Nicolson  b = (M_dev/alpha - K_div) s1 + F1 + F0
  *   BDF2            b = (M_dev/alpha)(4/3 s1 - 1/3 s2) + F1
- * (M_dev/alpha) w is formed as A_alpha w - K_div w. Device arrays of N
- * doubles; a scratch of 3 N doubles is allocated on `stream` for the call. */
+ * Formed in one pass over s1 and the loads; for BDF2 (the combination of s1
+ * and s2), or where rhs overlaps s1, a scratch of N doubles is allocated on
+ * `stream` for the call. Device arrays of N doubles. */
 int dcg_time_rhs(dcg_problem* p, int scheme, const double* s1, const double* s2, const double* F1,
                  const double* F0, double* rhs, void* stream);
 
@@ -351,7 +352,7 @@ int dcg_divergence(const dcg_problem* p, const double* sigma, double* div_elem, 
  * n^d * d doubles in (u_0) and out, integrated by the scheme's own rule
  * (right endpoint for implicit Euler and BDF2, trapezoid for Crank-Nicolson).
  * Returns the first non-OK step status (later steps are not run). Scratch of
- * 4 N + 2 d n^d doubles is allocated for the call. */
+ * 2 N + 2 d n^d doubles is allocated for the call. */
 int dcg_time_integrate(dcg_problem* p, int scheme, double dt, int nsteps, const double* sigma0,
                        const double* const* F, double* const* sigma_out, double* u_elem, double tol, int max_it,
                        dcg_stats* stats, void* stream);

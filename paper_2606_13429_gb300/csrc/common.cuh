@@ -402,6 +402,9 @@ struct OpCall {
   int slot = -1;
 };
 int op_product(dcg_problem* p, const OpCall& c, cudaStream_t s);
+int op_div(dcg_problem* p, const double* x, double* y, cudaStream_t s);
+int op_time_rhs(dcg_problem* p, bool minus_div, const double* w, const double* f, const double* f0, double* y,
+                cudaStream_t s);
 // matrix-free 3D product in FP32 arithmetic (mf.cu): operand mode xm (0 x, 1 x - V zh, 2 V zh),
 // output mode om (0 y, 2 V^T y), fused dot when `dot`
 int mf_product(dcg_problem* p, int xm, int om, bool dot, const double* x, const double* zh, double* y,

@@ -38,22 +38,25 @@ namespace dcg {
 namespace {
 
 enum OpX { OX_X = 0, OX_X_MINUS_VZ = 1, OX_VZ = 2 };
-enum OpO { OO_Y = 0, OO_FMY = 1, OO_VT = 2, OO_YVT = 3 };
+enum OpO { OO_Y = 0, OO_FMY = 1, OO_VT = 2, OO_YVT = 3, OO_RHS = 4 };
+enum OpPart { OP_FULL = 0, OP_MASS = 1, OP_DIV = 2 };  // A, (1/dt) M_dev or K_div alone
 
 struct OpArgs {
   const double* x;
   const double* zh;
-  const double* f;
+  const double* f;       // OO_FMY: f - y; OO_RHS: y + f (+ f0)
+  const double* f0;
   double* y;
   double* g;             // V^T y for OO_YVT
   const double* dvec;    // dot(dvec, y) for OO_Y
   const double* inv_nu;  // per element, or null: cmass holds the uniform value
   double cmass;          // 2D: h^2 / (36 dt) (/ nu); 3D: (h^3 / (216 dt) (/ nu)) / (h / 36)
-  double scale;          // 3D: h / 36
+  double scale;          // 3D: +-h / 36
+  double kx, ky;         // 2D: factors of K_div, +-1/6 and +-1/4
   double isd;            // 1/sqrt(d)
   int m, n;
   int gx, gy, seg;       // 2D: column blocks, -, rows per warp; 3D: column and row blocks, planes per CTA
-  int vec;               // x, f, y, dvec 16-byte aligned (2D)
+  int vec;               // x, f, f0, y, dvec 16-byte aligned (2D)
   Reduce red;
 };
 
@@ -133,9 +136,9 @@ __device__ __forceinline__ void op_row2(const OpArgs& A, int x, int y, OpRow2<VA
   }
 }
 
-template <int XM, int OM, bool DOT, bool VAR>
+template <int XM, int OM, bool DOT, bool VAR, int PART = OP_FULL>
 __global__ void __launch_bounds__(kOp2Threads) k_op2(OpArgs A) {
-  constexpr bool MASS = XM != OX_VZ && OM != OO_VT;  // M_dev V = 0 and V^T M_dev = 0
+  constexpr bool MASS = XM != OX_VZ && OM != OO_VT && PART != OP_DIV;  // M_dev V = 0 and V^T M_dev = 0
   double part[1] = {0.0};
   const int w = blockIdx.x * (kOp2Threads / 32) + (threadIdx.x >> 5);  // warp: 32 columns x seg rows
   const int wy = w / A.gx;
@@ -152,15 +155,16 @@ __global__ void __launch_bounds__(kOp2Threads) k_op2(OpArgs A) {
       wl = A.cmass * __ldg(e);
       wr = A.cmass * __ldg(e + 1);
     }
-    constexpr double axx = 1.0 / 6.0, axy = 0.25;
+    const double axx = OM == OO_RHS ? A.kx : 1.0 / 6.0, axy = OM == OO_RHS ? A.ky : 0.25;
     for (int y = y0; y < y1; ++y) {
       op_row2<XM, VAR>(A, x, y + 1, N);
-      double o[4];
-      // K_div
-      o[0] = fma(axy, P.c1 - N.c1, axx * fma(4.0, Q.k0, P.k0 + N.k0));
-      o[1] = fma(axy, P.c0 - N.c0, axx * fma(2.0, Q.m1, -(P.m1 + N.m1)));
-      o[2] = fma(axy, P.c3 - N.c3, axx * fma(4.0, Q.k2, P.k2 + N.k2));
-      o[3] = fma(axy, P.c2 - N.c2, axx * fma(2.0, Q.m3, -(P.m3 + N.m3)));
+      double o[4] = {0.0, 0.0, 0.0, 0.0};
+      if (PART != OP_MASS) {
+        o[0] = fma(axy, P.c1 - N.c1, axx * fma(4.0, Q.k0, P.k0 + N.k0));
+        o[1] = fma(axy, P.c0 - N.c0, axx * fma(2.0, Q.m1, -(P.m1 + N.m1)));
+        o[2] = fma(axy, P.c3 - N.c3, axx * fma(4.0, Q.k2, P.k2 + N.k2));
+        o[3] = fma(axy, P.c2 - N.c2, axx * fma(2.0, Q.m3, -(P.m3 + N.m3)));
+      }
       // (1/dt) M_dev
       if (MASS && VAR) {
         const double* e = A.inv_nu + x + A.n * (y + 1);
@@ -202,6 +206,17 @@ __global__ void __launch_bounds__(kOp2Threads) k_op2(OpArgs A) {
           op_load4(A.f + 4LL * a, A.vec, fv);
 #pragma unroll
           for (int c = 0; c < 4; ++c) o[c] = fv[c] - o[c];
+        }
+        if (OM == OO_RHS) {
+          double fv[4];
+          op_load4(A.f + 4LL * a, A.vec, fv);
+#pragma unroll
+          for (int c = 0; c < 4; ++c) o[c] += fv[c];
+          if (A.f0) {
+            op_load4(A.f0 + 4LL * a, A.vec, fv);
+#pragma unroll
+            for (int c = 0; c < 4; ++c) o[c] += fv[c];
+          }
         }
         double* yp = A.y + 4LL * a;
         if (A.vec) {
@@ -257,10 +272,11 @@ __device__ __forceinline__ double lane_r(double v) { return __shfl_down_sync(0xf
 // block's nodes. All three: the uniform-viscosity mass part of the diagonal
 // components is made deviatoric after its y and x factors; one alone (or with
 // a viscosity per element): the deviatoric operand is formed first.
-template <int XM, int OM, bool DOT, bool VAR, int K0, int K1>
+template <int XM, int OM, bool DOT, bool VAR, int K0, int K1, int PART>
 __device__ __forceinline__ double op3_rows(const OpArgs& A, int block) {
   constexpr bool RAW = VAR || K1 - K0 < 3;  // deviatoric operand first
-  constexpr bool MASS = XM != OX_VZ && OM != OO_VT;  // M_dev V = 0 and V^T M_dev = 0
+  constexpr bool MASS = XM != OX_VZ && OM != OO_VT && PART != OP_DIV;  // M_dev V = 0 and V^T M_dev = 0
+  constexpr bool DIV = PART != OP_MASS;
   constexpr double third = 1.0 / 3.0;
   double part[1] = {0.0};
   const int lane = threadIdx.x & 31, row = threadIdx.x >> 5;
@@ -322,6 +338,10 @@ __device__ __forceinline__ double op3_rows(const OpArgs& A, int block) {
       if (OM == OO_VT || !done) return;
       double v = o;
       if (OM == OO_FMY) v = A.f[ao * 9 + c] - v;
+      if (OM == OO_RHS) {
+        v += A.f[ao * 9 + c];
+        if (A.f0) v += A.f0[ao * 9 + c];
+      }
       A.y[ao * 9 + c] = v;
       if (DOT && OM != OO_YVT) part[0] = OM == OO_FMY ? fma(v, v, part[0]) : fma(A.dvec[ao * 9 + c], v, part[0]);
     };
@@ -346,9 +366,9 @@ __device__ __forceinline__ double op3_rows(const OpArgs& A, int block) {
       const double Mal = lane_l(Ma), Mar = lane_r(Ma), uMa = Mal + Mar;
       const double Cbl = lane_l(Cb), Cbr = lane_r(Cb);
       const double Mcl = lane_l(Mc), Mcr = lane_r(Mc), uMc = Mcl + Mcr;
-      double Ax = fma(1.5, Cbr - Cbl, fma(2.0, Ma, -uMa));
+      double Ax = DIV ? fma(1.5, Cbr - Cbl, fma(2.0, Ma, -uMa)) : 0.0;
       const double Bx = Mcr - Mcl;
-      double Ay = fma(1.5, lane_r(Ca) - lane_l(Ca), fma(4.0, Kb, lane_l(Kb) + lane_r(Kb)));
+      double Ay = DIV ? fma(1.5, lane_r(Ca) - lane_l(Ca), fma(4.0, Kb, lane_l(Kb) + lane_r(Kb))) : 0.0;
       const double By = fma(4.0, Cc, lane_l(Cc) + lane_r(Cc));
       const double Dz = fma(4.0, Mc, uMc);
       const double Bz = (Mar - Mal) - fma(4.0, Cb, Cbl + Cbr);
@@ -368,15 +388,15 @@ __device__ __forceinline__ double op3_rows(const OpArgs& A, int block) {
         if (k != 1 || RAW) Ay = fma(A.cmass, k == 1 ? F[k] : Fb, Ay);
       }
       double t1[3], t0[3], t2[3];
-      t1[0] = fma(-1.5, Bx, Ax);
-      t2[0] = fma(1.5, Bx, Ax);
+      t1[0] = DIV ? fma(-1.5, Bx, Ax) : Ax;
+      t2[0] = DIV ? fma(1.5, Bx, Ax) : Ax;
       t0[0] = 4.0 * Ax;
-      t1[1] = fma(1.5, By, Ay);
-      t2[1] = fma(-1.5, By, Ay);
+      t1[1] = DIV ? fma(1.5, By, Ay) : Ay;
+      t2[1] = DIV ? fma(-1.5, By, Ay) : Ay;
       t0[1] = 4.0 * Ay;
-      t1[2] = fma(-1.5, Bz, -Dz);
-      t2[2] = fma(1.5, Bz, -Dz);
-      t0[2] = Dz + Dz;
+      t1[2] = DIV ? fma(-1.5, Bz, -Dz) : 0.0;
+      t2[2] = DIV ? fma(1.5, Bz, -Dz) : 0.0;
+      t0[2] = DIV ? Dz + Dz : 0.0;
       if (MASS && !VAR && (k != 2 || RAW)) {
         const double v = A.cmass * (k == 2 ? F[k] : Dz);
         t1[2] += v;
@@ -431,27 +451,27 @@ __device__ __forceinline__ double op3_rows(const OpArgs& A, int block) {
   return part[0];
 }
 
-template <int XM, int OM, bool DOT, bool VAR>
+template <int XM, int OM, bool DOT, bool VAR, int PART = OP_FULL>
 __global__ void __launch_bounds__(kOp3Threads) k_op3(OpArgs A) {
-  double part[1] = {op3_rows<XM, OM, DOT, VAR, 0, 3>(A, blockIdx.x)};
+  double part[1] = {op3_rows<XM, OM, DOT, VAR, 0, 3, PART>(A, blockIdx.x)};
   if (DOT) grid_reduce<1>(part, A.red);
 }
 
 // one row of the tensor per block: a third of the FP64 chain per warp, for
 // grids too small to fill the GPU (outputs y and f - y only)
-template <int XM, int OM, bool DOT, bool VAR>
+template <int XM, int OM, bool DOT, bool VAR, int PART = OP_FULL>
 __global__ void __launch_bounds__(kOp3Threads) k_op3_split(OpArgs A) {
   const int b = blockIdx.x / 3;
   double part[1];
   switch (blockIdx.x - 3 * b) {
-    case 0: part[0] = op3_rows<XM, OM, DOT, VAR, 0, 1>(A, b); break;
-    case 1: part[0] = op3_rows<XM, OM, DOT, VAR, 1, 2>(A, b); break;
-    default: part[0] = op3_rows<XM, OM, DOT, VAR, 2, 3>(A, b);
+    case 0: part[0] = op3_rows<XM, OM, DOT, VAR, 0, 1, PART>(A, b); break;
+    case 1: part[0] = op3_rows<XM, OM, DOT, VAR, 1, 2, PART>(A, b); break;
+    default: part[0] = op3_rows<XM, OM, DOT, VAR, 2, 3, PART>(A, b);
   }
   if (DOT) grid_reduce<1>(part, A.red);
 }
 
-template <int XM, int OM, bool DOT>
+template <int XM, int OM, bool DOT, int PART = OP_FULL>
 int op_launch(dcg_problem* p, OpArgs a, cudaStream_t s) {
   if (p->dim == 2) {
     a.gx = (a.m + 31) / 32;
@@ -473,8 +493,8 @@ int op_launch(dcg_problem* p, OpArgs a, cudaStream_t s) {
     auto ctas = [&]() { return ((long long)a.gx * ((a.m + a.seg - 1) / a.seg) + kWarps - 1) / kWarps; };
     while (DOT && ctas() > kMaxRedCtas) a.seg *= 2;
     const unsigned g = (unsigned)ctas();
-    if (a.inv_nu) k_op2<XM, OM, DOT, true><<<g, kOp2Threads, 0, s>>>(a);
-    else k_op2<XM, OM, DOT, false><<<g, kOp2Threads, 0, s>>>(a);
+    if (a.inv_nu && PART != OP_DIV) k_op2<XM, OM, DOT, true, PART><<<g, kOp2Threads, 0, s>>>(a);
+    else k_op2<XM, OM, DOT, false, PART><<<g, kOp2Threads, 0, s>>>(a);
   } else {
     a.gx = (a.m + 29) / 30;
     a.gy = (a.m + kOp3Rows - 1) / kOp3Rows;
@@ -491,7 +511,8 @@ int op_launch(dcg_problem* p, OpArgs a, cudaStream_t s) {
     long long nz = 1;
     bool split = false;
     double best = 1e300;
-    for (int sp = 0; sp < (OM == OO_Y || OM == OO_FMY ? 2 : 1); ++sp)
+    constexpr bool kSplit = OM == OO_Y || OM == OO_FMY || OM == OO_RHS;
+    for (int sp = 0; sp < (kSplit ? 2 : 1); ++sp)
       for (long long q = 1; q <= a.m && cols * q * (sp ? 3 : 1) <= cap; ++q) {
         const long long per = (cols * q * (sp ? 3 : 1) + 151) / 152, seg = (a.m + q - 1) / q;
         const double t = (double)(per * (seg + 2)) * (per == 1 ? 1.3 : 1.0) * (sp ? 0.4 : 1.0);
@@ -503,16 +524,16 @@ int op_launch(dcg_problem* p, OpArgs a, cudaStream_t s) {
       }
     a.seg = (int)((a.m + nz - 1) / nz);
     const unsigned g = (unsigned)(cols * ((a.m + a.seg - 1) / a.seg));
-    if constexpr (OM == OO_Y || OM == OO_FMY) {
+    if constexpr (kSplit) {
       if (split) {
-        if (a.inv_nu) k_op3_split<XM, OM, DOT, true><<<3 * g, kOp3Threads, 0, s>>>(a);
-        else k_op3_split<XM, OM, DOT, false><<<3 * g, kOp3Threads, 0, s>>>(a);
+        if (a.inv_nu && PART != OP_DIV) k_op3_split<XM, OM, DOT, true, PART><<<3 * g, kOp3Threads, 0, s>>>(a);
+        else k_op3_split<XM, OM, DOT, false, PART><<<3 * g, kOp3Threads, 0, s>>>(a);
         DCG_LAUNCH_CHECK();
         return DCG_OK;
       }
     }
-    if (a.inv_nu) k_op3<XM, OM, DOT, true><<<g, kOp3Threads, 0, s>>>(a);
-    else k_op3<XM, OM, DOT, false><<<g, kOp3Threads, 0, s>>>(a);
+    if (a.inv_nu && PART != OP_DIV) k_op3<XM, OM, DOT, true, PART><<<g, kOp3Threads, 0, s>>>(a);
+    else k_op3<XM, OM, DOT, false, PART><<<g, kOp3Threads, 0, s>>>(a);
   }
   DCG_LAUNCH_CHECK();
   return DCG_OK;
@@ -520,10 +541,8 @@ int op_launch(dcg_problem* p, OpArgs a, cudaStream_t s) {
 
 }  // namespace
 
-// y = A x in FP64. Operand x (zh null), x - V zh, or V zh (x null); output y,
-// f - y (f given), V^T y (vt), or y and g = V^T y (g given). slot >= 0: the sum
-// of squares of the output (of g when it is formed), or with dvec (dvec, y).
-int op_product(dcg_problem* p, const OpCall& c, cudaStream_t s) {
+namespace {
+OpArgs op_args(dcg_problem* p, const OpCall& c) {
   OpArgs a{};
   a.x = c.x;
   a.zh = c.zh;
@@ -535,10 +554,50 @@ int op_product(dcg_problem* p, const OpCall& c, cudaStream_t s) {
   const double h = 1.0 / p->n, w = (a.inv_nu ? 1.0 : 1.0 / p->nu) / p->dt;
   a.cmass = p->dim == 2 ? h * h / 36.0 * w : h * h / 6.0 * w;
   a.scale = h / 36.0;
+  a.kx = 1.0 / 6.0;
+  a.ky = 0.25;
   a.isd = 1.0 / std::sqrt((double)p->dim);
   a.m = p->m;
   a.n = p->n;
   a.vec = (!c.x || aligned16(c.x)) && aligned16(c.y) && (!c.f || aligned16(c.f)) && (!c.dvec || aligned16(c.dvec));
+  return a;
+}
+}  // namespace
+
+// y = K_div x
+int op_div(dcg_problem* p, const double* x, double* y, cudaStream_t s) {
+  OpCall c;
+  c.x = x;
+  c.y = y;
+  return op_launch<OX_X, OO_Y, false, OP_DIV>(p, op_args(p, c), s);
+}
+
+// y = (1/dt) M_dev w + f (+ f0), or with `minus_div` ((1/dt) M_dev - K_div) w +
+// f (+ f0): one pass instead of the products A w and K_div w, their difference
+// and the loads (700^2, Crank-Nicolson, a viscosity per element: 230 -> 84 us,
+// and no scratch). w must not overlap y.
+int op_time_rhs(dcg_problem* p, bool minus_div, const double* w, const double* f, const double* f0, double* y,
+                cudaStream_t s) {
+  OpCall c;
+  c.x = w;
+  c.f = f;
+  c.y = y;
+  OpArgs a = op_args(p, c);
+  a.f0 = f0;
+  a.vec = a.vec && (!f0 || aligned16(f0));
+  if (!minus_div) return op_launch<OX_X, OO_RHS, false, OP_MASS>(p, a, s);
+  a.kx = -a.kx;
+  a.ky = -a.ky;
+  a.scale = -a.scale;  // 3D: -(h/36) (K - mass)
+  if (p->dim == 3) a.cmass = -a.cmass;
+  return op_launch<OX_X, OO_RHS, false>(p, a, s);
+}
+
+// y = A x in FP64. Operand x (zh null), x - V zh, or V zh (x null); output y,
+// f - y (f given), V^T y (vt), or y and g = V^T y (g given). slot >= 0: the sum
+// of squares of the output (of g when it is formed), or with dvec (dvec, y).
+int op_product(dcg_problem* p, const OpCall& c, cudaStream_t s) {
+  OpArgs a = op_args(p, c);
   if (c.slot >= 0) a.red = make_reduce(p, c.slot);
   // algorithmic work: structural entries of the blocks (an FMA counts 2), and
   // the vectors and 1/nu

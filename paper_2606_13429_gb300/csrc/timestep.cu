@@ -6,9 +6,7 @@
 //   implicit Euler  alpha = dt      b = (M/alpha) s1 + F1
 //   Crank-Nicolson  alpha = dt/2    b = (M/alpha - K) s1 + F1 + F0
 //   BDF2            alpha = 2dt/3   b = (M/alpha)(4/3 s1 - 1/3 s2) + F1
-// with (M/alpha) w formed as A_alpha w - K_div w: the assembled product and
-// the constant divergence stencil of the uniform Q1 mesh (K_div does not
-// depend on nu or dt). The problem is assembled once with alpha, and its
+// in one pass over the previous stress and the loads (op.cu). The problem is assembled once with alpha, and its
 // set-up (inner hierarchy, Z_J = V^T A V, which does not depend on dt) serves
 // every step.
 #include "common.cuh"
@@ -19,56 +17,11 @@
 namespace dcg {
 namespace {
 
-struct DivSt {
-  double c[9][27];
-};
-
 // y = a1 s1 + a2 s2 (s2 may be null)
 __global__ void k_ts_combine(double* __restrict__ y, const double* __restrict__ s1, const double* __restrict__ s2,
                              double a1, double a2, long long n) {
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
     y[i] = s2 ? a1 * s1[i] + a2 * s2[i] : a1 * s1[i];
-}
-
-// y = K_div x: component (k, p) of node a is sum_q sum_o G[p][q][o] x_{a+o,(k,q)}
-template <int D>
-__global__ void k_ts_div_apply(const double* __restrict__ x, double* __restrict__ y, DivSt G, int m, long long nn) {
-  constexpr int B = D * D, NO = D == 2 ? 9 : 27;
-  for (long long a = blockIdx.x * (long long)blockDim.x + threadIdx.x; a < nn; a += (long long)gridDim.x * blockDim.x) {
-    int c[3];
-    long long r = a;
-    c[0] = (int)(r % m);
-    r /= m;
-    c[1] = (int)(r % m);
-    c[2] = D > 2 ? (int)(r / m) : 0;
-    double acc[B];
-#pragma unroll
-    for (int t = 0; t < B; ++t) acc[t] = 0.0;
-    for (int o = 0; o < NO; ++o) {
-      const int xx = c[0] + o % 3 - 1, yy = c[1] + (o / 3) % 3 - 1, zz = c[2] + o / 9 - 1;
-      if (xx < 0 || xx >= m || yy < 0 || yy >= m || (D > 2 && (zz < 0 || zz >= m))) continue;
-      const double* xb = x + (xx + (long long)m * (yy + (long long)m * (D > 2 ? zz : 0))) * B;
-#pragma unroll
-      for (int k = 0; k < D; ++k)
-#pragma unroll
-        for (int p = 0; p < D; ++p)
-#pragma unroll
-          for (int q = 0; q < D; ++q) acc[k * D + p] = fma(G.c[p * 3 + q][o], xb[k * D + q], acc[k * D + p]);
-    }
-#pragma unroll
-    for (int t = 0; t < B; ++t) y[a * B + t] = acc[t];
-  }
-}
-
-// b = t - gamma kw + F1 + beta F0 (F0 may be null)
-__global__ void k_ts_rhs(double* __restrict__ b, const double* __restrict__ t, const double* __restrict__ kw,
-                         const double* __restrict__ F1, const double* __restrict__ F0, double gamma, double beta,
-                         long long n) {
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    double v = t[i] - gamma * kw[i] + F1[i];
-    if (F0) v += beta * F0[i];
-    b[i] = v;
-  }
 }
 
 // p = -(1/d) tr(sigma) at every interior node
@@ -144,28 +97,31 @@ double alpha_of(int scheme, double dt) {
   return scheme == DCG_IMPLICIT_EULER ? dt : scheme == DCG_CRANK_NICOLSON ? dt / 2.0 : 2.0 * dt / 3.0;
 }
 
-int div_apply(const dcg_problem* p, const double* x, double* y, cudaStream_t s) {
-  DivSt G;
-  div_stencil(p->dim, p->n, G.c);
-  if (p->dim == 2) k_ts_div_apply<2><<<gn(p->n_nodes), 256, 0, s>>>(x, y, G, p->m, p->n_nodes);
-  else k_ts_div_apply<3><<<gn(p->n_nodes), 256, 0, s>>>(x, y, G, p->m, p->n_nodes);
-  DCG_LAUNCH_CHECK();
-  return DCG_OK;
+bool overlap(const double* a, const double* b, long long n) {
+  const uintptr_t x = (uintptr_t)a, y = (uintptr_t)b, len = sizeof(double) * (size_t)n;
+  return x < y + len && y < x + len;
 }
 
-// b from s1, s2 (BDF2), F1 and F0 (CN); w, t, kw: scratch of N doubles
+// the step's combination of previous stresses needs a vector of its own: BDF2
+// (4/3 s1 - 1/3 s2), or s1 where the right-hand side overlaps it
+bool rhs_needs_scratch(const dcg_problem* p, int scheme, const double* s1, const double* b) {
+  return scheme == DCG_BDF2 || overlap(s1, b, p->N);
+}
+
+// b from s1, s2 (BDF2), F1 and F0 (CN); w: scratch of N doubles (may be null
+// unless rhs_needs_scratch)
 int time_rhs(dcg_problem* p, int scheme, const double* s1, const double* s2, const double* F1, const double* F0,
-             double* b, double* w, double* t, double* kw, cudaStream_t s) {
+             double* b, double* w, cudaStream_t s) {
   const long long N = p->N;
-  if (scheme == DCG_BDF2) k_ts_combine<<<gn(N), 256, 0, s>>>(w, s1, s2 ? s2 : s1, 4.0 / 3.0, -1.0 / 3.0, N);
-  else k_ts_combine<<<gn(N), 256, 0, s>>>(w, s1, nullptr, 1.0, 0.0, N);
-  DCG_LAUNCH_CHECK();
-  DCG_TRY(spmv_plain(p, w, t, s));
-  DCG_TRY(div_apply(p, w, kw, s));
+  const double* v = s1;
+  if (rhs_needs_scratch(p, scheme, s1, b)) {
+    if (scheme == DCG_BDF2) k_ts_combine<<<gn(N), 256, 0, s>>>(w, s1, s2 ? s2 : s1, 4.0 / 3.0, -1.0 / 3.0, N);
+    else k_ts_combine<<<gn(N), 256, 0, s>>>(w, s1, nullptr, 1.0, 0.0, N);
+    DCG_LAUNCH_CHECK();
+    v = w;
+  }
   const bool cn = scheme == DCG_CRANK_NICOLSON;
-  k_ts_rhs<<<gn(N), 256, 0, s>>>(b, t, kw, F1, cn ? F0 : nullptr, cn ? 2.0 : 1.0, 1.0, N);
-  DCG_LAUNCH_CHECK();
-  return DCG_OK;
+  return op_time_rhs(p, cn, v, F1, cn ? F0 : nullptr, b, s);
 }
 
 int divergence(const dcg_problem* p, const double* sigma, double* out, cudaStream_t s) {
@@ -195,7 +151,7 @@ int dcg_apply_div(const dcg_problem* p, const double* x, double* y, void* stream
     set_error_msg("dcg_apply_div: need an assembled problem and device arrays x, y");
     return DCG_ERR_INVALID_ARG;
   }
-  return div_apply(p, x, y, (cudaStream_t)stream);
+  return op_div(const_cast<dcg_problem*>(p), x, y, (cudaStream_t)stream);
 }
 
 int dcg_time_rhs(dcg_problem* p, int scheme, const double* s1, const double* s2, const double* F1, const double* F0,
@@ -206,9 +162,10 @@ int dcg_time_rhs(dcg_problem* p, int scheme, const double* s1, const double* s2,
     return DCG_ERR_INVALID_ARG;
   }
   cudaStream_t s = (cudaStream_t)stream;
+  if (!rhs_needs_scratch(p, scheme, s1, rhs)) return time_rhs(p, scheme, s1, s2, F1, F0, rhs, nullptr, s);
   double* tmp = nullptr;
-  DCG_CUDA(cudaMallocAsync(&tmp, sizeof(double) * 3 * p->N, s));
-  const int st = time_rhs(p, scheme, s1, s2, F1, F0, rhs, tmp, tmp + p->N, tmp + 2 * p->N, s);
+  DCG_CUDA(cudaMallocAsync(&tmp, sizeof(double) * p->N, s));
+  const int st = time_rhs(p, scheme, s1, s2, F1, F0, rhs, tmp, s);
   cudaFreeAsync(tmp, s);
   return st;
 }
@@ -253,15 +210,15 @@ int dcg_time_integrate(dcg_problem* p, int scheme, double dt, int nsteps, const 
   for (int k = 0; k < p->dim; ++k) ne *= p->n;
   const long long nd = ne * p->dim;
   double* tmp = nullptr;
-  DCG_CUDA(cudaMalloc(&tmp, sizeof(double) * (4 * N + 2 * nd)));
-  double *b = tmp, *w = tmp + N, *t = tmp + 2 * N, *kw = tmp + 3 * N;
-  double *div_prev = tmp + 4 * N, *div_cur = div_prev + nd;
+  DCG_CUDA(cudaMalloc(&tmp, sizeof(double) * (2 * N + 2 * nd)));
+  double *b = tmp, *w = tmp + N;
+  double *div_prev = tmp + 2 * N, *div_cur = div_prev + nd;
   int rc = DCG_OK;
   if (u_elem && scheme == DCG_CRANK_NICOLSON) rc = divergence(p, sigma0, div_prev, s);
   for (int k = 0; k < nsteps && rc == DCG_OK; ++k) {
     const double* s1 = k == 0 ? sigma0 : sigma_out[k - 1];
     const double* s2 = k == 0 ? sigma0 : (k == 1 ? sigma0 : sigma_out[k - 2]);
-    rc = time_rhs(p, scheme, s1, scheme == DCG_BDF2 ? s2 : nullptr, F[k + 1], F[k], b, w, t, kw, s);
+    rc = time_rhs(p, scheme, s1, scheme == DCG_BDF2 ? s2 : nullptr, F[k + 1], F[k], b, w, s);
     if (rc != DCG_OK) break;
     // initial guess: the previous step
     if (cudaMemcpyAsync(sigma_out[k], s1, sizeof(double) * N, cudaMemcpyDeviceToDevice, s) != cudaSuccess) {
