@@ -190,7 +190,8 @@ struct Level {
   Stencil<double> st64{};
   Stencil<float> st32{};
   // 2D stencil with 8 equal neighbour coefficients (the Q1 Laplacian):
-  // Z z = box_c0 z + box_c1 (3 x 3 box sum), box_c0 = centre - box_c1
+  // Z z = box_c0 z + box_c1 (3 x 3 box sum), box_c0 = centre - box_c1; 3D
+  // stencil with faces 0, edges 2 box_c1, corners box_c1, centre box_c0
   bool box = false;
   double box_c0 = 0.0, box_c1 = 0.0;
   // RAS

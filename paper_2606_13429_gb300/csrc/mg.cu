@@ -374,11 +374,17 @@ __global__ void k_residual(Stencil<T> st, const T* __restrict__ f, const T* __re
 // with the box sum formed from row sums s(y) = z(x-1,y) + z(x,y) + z(x+1,y)
 // that slide along y: a residual takes 4 additions and 2 FMAs per node
 // instead of 9 FMAs and a subtraction (FP64 issue is what the FP64 cycle
-// spends). A thread walks kBoxSeg rows of one column; consecutive threads
+// spends). A thread walks SEG rows of one column; consecutive threads
 // take consecutive columns, so every row access is coalesced. Entries
-// outside the grid are zero (Dirichlet nodes eliminated).
-constexpr int kBoxSeg = 8;
+// outside the grid are zero (Dirichlet nodes eliminated). SEG is 8 where that
+// gives each SM four CTAs (1023^2: 1,024 CTAs, FP64 issue is the bound and the
+// two extra row sums per segment its overhead), else 2: a small grid waits
+// for the serial walk (495^2 in FP32: 8.5 us with 8 rows, 5.1 us with 2).
 constexpr int kBoxThreads = 128;
+inline int box_seg(int m) {
+  const long long gx = (m + kBoxThreads - 1) / kBoxThreads;
+  return gx * ((m + 7) / 8) >= 4 * 152 ? 8 : 2;
+}
 
 template <typename T>
 __device__ __forceinline__ T box_row(const T* __restrict__ z, int x, int y, int m, T& centre) {
@@ -392,14 +398,14 @@ __device__ __forceinline__ T box_row(const T* __restrict__ z, int x, int y, int 
   return s;
 }
 
-// Walks rows y0 .. y0 + kBoxSeg - 1 of column x and calls
+// Walks rows y0 .. y0 + SEG - 1 of column x and calls
 // body(a, r_a) with r_a = f_a - (Z z)_a. Rows are loaded kBoxU at a time
 // (all their loads in flight together) before the sums slide over them.
-constexpr int kBoxU = 4;
-template <typename T, typename F, typename Body>
+template <int SEG, typename T, typename F, typename Body>
 __device__ __forceinline__ void box_residual_walk(T c0, T c1, const F* __restrict__ f, const T* __restrict__ z, int m,
                                                   int x, int y0, Body&& body) {
-  const int y1 = min(y0 + kBoxSeg, m);
+  constexpr int kBoxU = SEG < 4 ? SEG : 4;
+  const int y1 = min(y0 + SEG, m);
   T cm, c0v;
   T sm = box_row(z, x, y0 - 1, m, cm);
   T s0 = box_row(z, x, y0, m, c0v);
@@ -423,13 +429,87 @@ __device__ __forceinline__ void box_residual_walk(T c0, T c1, const F* __restric
   }
 }
 
-// y = f - Z z on a box-sum level (grid: columns / kBoxThreads x rows / kBoxSeg)
-template <typename T>
+// y = f - Z z on a box-sum level (grid: columns / kBoxThreads x rows / SEG)
+template <typename T, int SEG>
 __global__ void __launch_bounds__(kBoxThreads) k_residual_box(T c0, T c1, const T* __restrict__ f,
                                                               const T* __restrict__ z, T* __restrict__ y, int m) {
   const int x = blockIdx.x * kBoxThreads + threadIdx.x;
   if (x >= m) return;
-  box_residual_walk<T, T>(c0, c1, f, z, m, x, blockIdx.y * kBoxSeg, [&](long long a, T r) { y[a] = r; });
+  box_residual_walk<SEG, T, T>(c0, c1, f, z, m, x, blockIdx.y * SEG, [&](long long a, T r) { y[a] = r; });
+}
+
+// 3D levels whose stencil is the Q1 Laplacian / d: the 6 face coefficients
+// vanish and the 12 edge coefficients are twice the 8 corner ones (c3), so
+//   (Z z)_a = c0 z_a + c3 (E_{k-1} + E_{k+1} + 2 D_k)
+// with D_k the sum of the four diagonal neighbours in plane k and
+// E_k = D_k + 2 (the four nearest ones). A thread takes two rows of one column
+// x and walks SEG planes; the x sums of four rows serve both rows, the plane
+// sums slide along z: 10 FP64 instructions per node and, for the two end
+// planes of a segment, 6 / SEG x 2 more, instead of 27 FMAs (FP64 issue is the
+// bound). 127^3: residual 99 us -> 53 us, the inner residual 116 us -> 67 us.
+// SEG is 8 where that gives each SM four CTAs, else 2, as in 2D: a smaller
+// grid waits for the serial walk (31^3: 15.5 us with 8 planes, 6.9 us with 2).
+constexpr int kBox3Threads = 128;
+
+// threads of a walk: columns x row pairs x segments
+inline long long box3_items(int m, int seg) { return (long long)m * ((m + 1) / 2) * ((m + seg - 1) / seg); }
+inline int box3_seg(int m) { return box3_items(m, 8) >= 4 * 152 * kBox3Threads ? 8 : 2; }
+
+template <int SEG, typename Body>
+__device__ __forceinline__ void box3_residual_walk(double c0, double c3, const double* __restrict__ f,
+                                                   const double* __restrict__ z, int m, unsigned item, Body&& body) {
+  const unsigned pairs = (unsigned)(m + 1) / 2, q = item / (unsigned)m;
+  const int x = (int)(item - q * (unsigned)m), y = 2 * (int)(q % pairs), k0 = SEG * (int)(q / pairs);
+  const int mm = m * m, k1 = min(k0 + SEG, m);
+  const bool xl = x > 0, xr = x + 1 < m;
+  const int col = x + m * (y - 1);
+  // plane k: the two rows' centre values, D and E
+  auto plane = [&](int k, double (&cv)[2], double (&D)[2], double (&E)[2]) {
+    double X[4], C[4];
+    const bool in = k >= 0 && k < m;
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      const bool row = in && y - 1 + r >= 0 && y - 1 + r < m;
+      const double* p = z + (col + m * r + mm * k);
+      const double l = row && xl ? __ldg(p - 1) : 0.0;
+      const double h = row && xr ? __ldg(p + 1) : 0.0;
+      C[r] = row ? __ldg(p) : 0.0;
+      X[r] = l + h;
+    }
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      cv[u] = C[u + 1];
+      D[u] = X[u] + X[u + 2];
+      E[u] = fma(2.0, X[u + 1] + (C[u] + C[u + 2]), D[u]);
+    }
+  };
+  double c[2], D[2], E0[2], E1[2], t[2], u2[2];
+  plane(k0 - 1, t, u2, E0);
+  plane(k0, c, D, E1);
+  for (int k = k0; k < k1; ++k) {
+    double cn[2], Dn[2], En[2];
+    const int a = col + m + mm * k;
+    const bool second = y + 1 < m;
+    const double f0 = __ldg(f + a), f1 = second ? __ldg(f + a + m) : 0.0;
+    plane(k + 1, cn, Dn, En);
+    body(a, f0, fma(-c3, fma(2.0, D[0], E0[0] + En[0]), fma(-c0, c[0], f0)));
+    if (second) body(a + m, f1, fma(-c3, fma(2.0, D[1], E0[1] + En[1]), fma(-c0, c[1], f1)));
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      E0[u] = E1[u];
+      E1[u] = En[u];
+      D[u] = Dn[u];
+      c[u] = cn[u];
+    }
+  }
+}
+
+template <int SEG>
+__global__ void __launch_bounds__(kBox3Threads) k_residual_box3(double c0, double c3, const double* __restrict__ f,
+                                                                const double* __restrict__ z, double* __restrict__ y,
+                                                                int m, unsigned items) {
+  const unsigned t = blockIdx.x * kBox3Threads + threadIdx.x;
+  if (t < items) box3_residual_walk<SEG>(c0, c3, f, z, m, t, [&](int a, double, double r) { y[a] = r; });
 }
 
 // coarse[I] = sum_al w(al) fine[2I+1+al]  (P^T), weights 1, 1/2, 1/4, 1/8:
@@ -1577,7 +1657,7 @@ __global__ void k_inner_residual(Stencil<double> st, const double* __restrict__ 
 
 // k_inner_residual on a 2D box-sum level; a 1D grid of column blocks x row
 // segments (bx fastest), so that the grid reduction sees gridDim.x CTAs
-template <typename T>
+template <typename T, int SEG>
 __global__ void __launch_bounds__(kBoxThreads) k_inner_residual_box(double c0, double c1, const double* __restrict__ g,
                                                                     const double* __restrict__ z, T* __restrict__ fJ,
                                                                     T* __restrict__ zJ, int m, int gx, Reduce red,
@@ -1587,7 +1667,7 @@ __global__ void __launch_bounds__(kBoxThreads) k_inner_residual_box(double c0, d
   const int bx = blockIdx.x % gx, by = blockIdx.x / gx;
   const int x = bx * kBoxThreads + threadIdx.x;
   if (x < m) {
-    box_residual_walk<double, double>(c0, c1, g, z, m, x, by * kBoxSeg, [&](long long a, double r) {
+    box_residual_walk<SEG, double, double>(c0, c1, g, z, m, x, by * SEG, [&](long long a, double r) {
       const T rt = (T)r;
       fJ[a] = rt;
       zJ[a] = (T)0;
@@ -1598,6 +1678,27 @@ __global__ void __launch_bounds__(kBoxThreads) k_inner_residual_box(double c0, d
       }
     });
   }
+  part[0] = (double)rr;
+  grid_reduce<2>(part, red);
+}
+
+// k_inner_residual on a 3D box-sum level
+template <typename T, int SEG>
+__global__ void __launch_bounds__(kBox3Threads) k_inner_residual_box3(double c0, double c3, const double* __restrict__ g,
+                                                                      const double* __restrict__ z, T* __restrict__ fJ,
+                                                                      T* __restrict__ zJ, int m, unsigned items,
+                                                                      Reduce red, bool with_g) {
+  double part[2] = {0.0, 0.0};
+  T rr = (T)0;
+  const unsigned t = blockIdx.x * kBox3Threads + threadIdx.x;
+  if (t < items)
+    box3_residual_walk<SEG>(c0, c3, g, z, m, t, [&](int a, double ga, double r) {
+      const T rt = (T)r;
+      fJ[a] = rt;
+      zJ[a] = (T)0;
+      rr = fma(rt, rt, rr);
+      if (with_g) part[1] = fma(ga, ga, part[1]);
+    });
   part[0] = (double)rr;
   grid_reduce<2>(part, red);
 }
@@ -1948,9 +2049,20 @@ Stencil<double> st_of<double>(const Level& L) { return L.st64; }
 template <typename T, int D>
 void level_residual(const Level& L, const T* f, const T* z, T* r, cudaStream_t s) {
   if (D == 2 && L.box) {
-    const dim3 grid((unsigned)((L.m + kBoxThreads - 1) / kBoxThreads), (unsigned)((L.m + kBoxSeg - 1) / kBoxSeg));
-    k_residual_box<T><<<grid, kBoxThreads, 0, s>>>((T)L.box_c0, (T)L.box_c1, f, z, r, L.m);
+    const int seg = box_seg(L.m);
+    const dim3 grid((unsigned)((L.m + kBoxThreads - 1) / kBoxThreads), (unsigned)((L.m + seg - 1) / seg));
+    if (seg == 8) k_residual_box<T, 8><<<grid, kBoxThreads, 0, s>>>((T)L.box_c0, (T)L.box_c1, f, z, r, L.m);
+    else k_residual_box<T, 2><<<grid, kBoxThreads, 0, s>>>((T)L.box_c0, (T)L.box_c1, f, z, r, L.m);
   } else {
+    if constexpr (D == 3 && sizeof(T) == 8) {
+      if (L.box) {
+        const int seg = box3_seg(L.m);
+        const unsigned items = (unsigned)box3_items(L.m, seg), grid = (items + kBox3Threads - 1) / kBox3Threads;
+        if (seg == 8) k_residual_box3<8><<<grid, kBox3Threads, 0, s>>>(L.box_c0, L.box_c1, f, z, r, L.m, items);
+        else k_residual_box3<2><<<grid, kBox3Threads, 0, s>>>(L.box_c0, L.box_c1, f, z, r, L.m, items);
+        return;
+      }
+    }
     k_residual<T, D><<<grid_for(L.nn, 256, 8192), 256, 0, s>>>(st_of<T>(L), f, z, r, L.m, L.nn);
   }
 }
@@ -2297,6 +2409,21 @@ int mg_setup(dcg_problem* p, cudaStream_t s) {
         L.box_c0 = L.st64.c[4] - c1;
       }
     }
+    // 3D: faces 0, edges 2 c3, corners c3, to the same 1e-12
+    if (D == 3 && L.m >= 3) {
+      auto dist = [](int k) { return abs(k % 3 - 1) + abs(k / 3 % 3 - 1) + abs(k / 9 - 1); };
+      double sum = 0.0, dev = 0.0;
+      for (int k = 0; k < 27; ++k)
+        if (dist(k) >= 2) sum += L.st64.c[k];
+      const double c3 = sum / 32.0;  // 12 edges of 2 c3, 8 corners of c3
+      for (int k = 0; k < 27; ++k)
+        if (dist(k) > 0) dev = std::max(dev, std::fabs(L.st64.c[k] - c3 * (dist(k) == 3 ? 1.0 : dist(k) == 2 ? 2.0 : 0.0)));
+      if (c3 != 0.0 && dev <= 1e-12 * std::fabs(c3)) {
+        L.box = true;
+        L.box_c1 = c3;
+        L.box_c0 = L.st64.c[13];
+      }
+    }
   }
   // coarsest: check the closed form the fast-diagonalisation solver assumes
   {
@@ -2449,10 +2576,21 @@ int inner_residual(dcg_problem* p, const double* g, const double* z, cudaStream_
   const int grid = grid_for(L.nn, 256, kRedGrid);
   Reduce red = make_reduce(p, S_TMP0);  // S_TMP0 <- ||r||^2, S_TMP1 <- ||g||^2
   const int prof = prof_begin(p, PC_INNER_RES, s);
-  const int gx = (L.m + kBoxThreads - 1) / kBoxThreads, gy = (L.m + kBoxSeg - 1) / kBoxSeg;
-  if (p->dim == 2 && L.box && (long long)gx * gy <= kMaxRedCtas)
-    k_inner_residual_box<T><<<gx * gy, kBoxThreads, 0, s>>>(L.box_c0, L.box_c1, g, z, (T*)L.f, (T*)L.z, L.m, gx, red,
-                                                            with_g);
+  const int seg = box_seg(L.m), gx = (L.m + kBoxThreads - 1) / kBoxThreads, gy = (L.m + seg - 1) / seg;
+  const int seg3 = box3_seg(L.m);
+  const long long items = box3_items(L.m, seg3), ctas = (items + kBox3Threads - 1) / kBox3Threads;
+  if (p->dim == 2 && L.box && (long long)gx * gy <= kMaxRedCtas && seg == 8)
+    k_inner_residual_box<T, 8><<<gx * gy, kBoxThreads, 0, s>>>(L.box_c0, L.box_c1, g, z, (T*)L.f, (T*)L.z, L.m, gx, red,
+                                                               with_g);
+  else if (p->dim == 2 && L.box && (long long)gx * gy <= kMaxRedCtas)
+    k_inner_residual_box<T, 2><<<gx * gy, kBoxThreads, 0, s>>>(L.box_c0, L.box_c1, g, z, (T*)L.f, (T*)L.z, L.m, gx, red,
+                                                               with_g);
+  else if (p->dim == 3 && L.box && ctas <= kMaxRedCtas && seg3 == 8)
+    k_inner_residual_box3<T, 8><<<(unsigned)ctas, kBox3Threads, 0, s>>>(L.box_c0, L.box_c1, g, z, (T*)L.f, (T*)L.z, L.m,
+                                                                        (unsigned)items, red, with_g);
+  else if (p->dim == 3 && L.box && ctas <= kMaxRedCtas)
+    k_inner_residual_box3<T, 2><<<(unsigned)ctas, kBox3Threads, 0, s>>>(L.box_c0, L.box_c1, g, z, (T*)L.f, (T*)L.z, L.m,
+                                                                        (unsigned)items, red, with_g);
   else if (p->dim == 2)
     k_inner_residual<T, 2><<<grid, 256, 0, s>>>(L.st64, g, z, (T*)L.f, (T*)L.z, nullptr, L.m, L.nn, red, with_g);
   else
