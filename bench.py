@@ -437,7 +437,7 @@ def run_ours(args):
 
     # SpMV bandwidth on this operator (FP64, plain product) and the per-class rooflines
     extra["spmv_fp64"] = spmv_rate(dcg, inputs, torch, n, peaks)
-    extra["class_rooflines"] = class_rooflines(breakdown, peaks, fp64_peak)
+    extra["class_rooflines"] = class_rooflines(breakdown, peaks, fp64_peak, fp32_peak)
     extra["kernel_breakdown_warmup_ms"] = {c: round(v["ms"], 3) for c, v in breakdown.items()}
     # the batched workload runs its multigrid in FP32 (BF16 inverses) with
     # FP64 outer CG; its options are autotuned per mesh size from these
@@ -452,7 +452,7 @@ def run_ours(args):
             extra[key] = {"error": "%s: %s" % (type(exc).__name__, exc)}
         torch.cuda.empty_cache()
 
-    roof = roofline(dominant, dom, peaks, peak_src, fp64_peak)
+    roof = roofline(dominant, dom, peaks, peak_src, fp64_peak, fp32_peak)
 
     cpu = None
     if rank == 0 and ws == 1 and not args.skip_cpu:
@@ -495,8 +495,9 @@ def run_ours(args):
 
 
 def spmv_rate(dcg, inputs, torch, n, peaks):
-    """The FP64 BSR product alone (20 launches after one warm-up): GB/s of the
-    algorithmic bytes against the measured copy bandwidth."""
+    """The FP64 product alone (20 launches after one warm-up): GB/s of the
+    algorithmic bytes (the vectors; large grids read no stored blocks) against
+    the measured copy bandwidth."""
     p = dcg.dcg_assemble(2, n, 1e-6)
     f = torch.from_numpy(inputs.rhs(0, p.N)).cuda()
     y = torch.empty_like(f)
@@ -512,10 +513,17 @@ def spmv_rate(dcg, inputs, torch, n, peaks):
             "algorithmic_bytes_per_launch": sp["bytes"] / max(1, sp["launches"])}
 
 
-def class_rooflines(breakdown, peaks, fp64_peak):
+def alu_peak(cls, fp64_peak, fp32_peak):
+    """Arithmetic roof (TFLOP/s) of a class of the FP64 solver. The smoother's
+    local solves run in 64-bit fixed point: a multiply-add is three wide
+    integer multiply-adds, each at half the measured FP32 FMA rate."""
+    return fp32_peak / 6.0 if cls == "ras_solve" else fp64_peak
+
+
+def class_rooflines(breakdown, peaks, fp64_peak, fp32_peak):
     """Per kernel class over the warm-up solves: algorithmic GB/s and TFLOP/s
-    against the measured HBM copy bandwidth and FP64 FMA rate; the roof of a
-    class is the smaller of the two times its work needs."""
+    against the measured HBM copy bandwidth and the class's arithmetic roof;
+    the roof of a class is the larger of the two times its work needs."""
     out = {}
     for c, v in breakdown.items():
         if v["ms"] <= 0:
@@ -524,9 +532,10 @@ def class_rooflines(breakdown, peaks, fp64_peak):
         gbs = v["bytes"] / secs / 1e9
         tf = v["flops"] / secs / 1e12
         t_hbm = v["bytes"] / (peaks["hbm_gbs"] * 1e9)
-        t_alu = v["flops"] / (fp64_peak * 1e12)
+        peak = alu_peak(c, fp64_peak, fp32_peak)
+        t_alu = v["flops"] / (peak * 1e12)
         out[c] = {"ms": round(v["ms"], 3), "launches": v["launches"], "GB_per_s": gbs, "TFLOP_per_s": tf,
-                  "frac_hbm": gbs / peaks["hbm_gbs"], "frac_fp64": tf / fp64_peak,
+                  "frac_hbm": gbs / peaks["hbm_gbs"], "frac_fp64": tf / fp64_peak, "frac_alu": tf / peak,
                   "frac_of_roof": max(t_hbm, t_alu) / secs}
     return out
 
@@ -652,12 +661,9 @@ def bsr3d_extra(args, opts, dcg, inputs, torch):
     y = torch.empty_like(f)
     sp_ms = _timed(torch, lambda: dcg.dcg_spmv(prob, f, y), 10)
     out["spmv_fp64_ms"] = sp_ms
-    # bytes of the product in the stored BSR format (81 values per block): the
-    # kernel skips the 48 structural zeros of a block, but DRAM still moves
-    # the whole blocks (ncu: DRAM reads equal the stored bytes), at a read
-    # rate above the copy bandwidth (which mixes reads and writes)
-    fmt = prob.nnzb * 81 * 8 + prob.nnzb * 4 + 2 * prob.N * 8
-    out["spmv_fp64_GB_per_s"] = fmt / (sp_ms * 1e-3) / 1e9
+    # bytes of the product in factored form: x in, y out (the stored blocks
+    # are not read; the product is bound by FP64 issue)
+    out["spmv_fp64_GB_per_s"] = 2 * prob.N * 8 / (sp_ms * 1e-3) / 1e9
     out["spmv_fp64_frac_of_copy_bw"] = out["spmv_fp64_GB_per_s"] / load_peaks()[0]["hbm_gbs"]
     prob.close()
     return out
@@ -760,10 +766,10 @@ def kernel_source_hash(files=None, functions=None):
     return h.hexdigest()[:16]
 
 
-def roofline(dominant, dom, peaks, peak_src, fp64_peak):
+def roofline(dominant, dom, peaks, peak_src, fp64_peak, fp32_peak):
     """Roofline of the dominant kernel class over the timed region: its
-    algorithmic bytes and FP64 flops against the measured HBM copy bandwidth
-    and the measured FP64 FMA rate; the bound is whichever needs more time."""
+    algorithmic bytes and flops against the measured HBM copy bandwidth and
+    the class's arithmetic roof; the bound is whichever needs more time."""
     secs = dom["ms"] / 1e3
     traffic = None
     try:
@@ -780,12 +786,15 @@ def roofline(dominant, dom, peaks, peak_src, fp64_peak):
     if secs <= 0:
         return dict(base, bound="hbm", achieved=0.0, peak=peaks["hbm_gbs"], unit="GB/s", frac=0.0)
     t_hbm = dom["bytes"] / (peaks["hbm_gbs"] * 1e9)
-    t_alu = dom["flops"] / (fp64_peak * 1e12)
+    peak = alu_peak(dominant, fp64_peak, fp32_peak)
+    t_alu = dom["flops"] / (peak * 1e12)
     if t_alu > t_hbm:
         achieved = dom["flops"] / secs / 1e12
-        return dict(base, bound="alu", achieved=achieved, peak=fp64_peak, unit="TFLOP/s", frac=achieved / fp64_peak,
-                    peak_source="FP64 FMA rate measured on this GPU by dcg_measure_fma_rate (independent FMA chains "
-                                "on all SMs); an FMA counts 2 flops")
+        src = ("FP32 FMA rate measured on this GPU by dcg_measure_fma_rate / 6 (64-bit fixed point: three wide integer "
+               "multiply-adds per multiply-add, at half the FP32 rate)" if dominant == "ras_solve" else
+               "FP64 FMA rate measured on this GPU by dcg_measure_fma_rate (independent FMA chains on all SMs)")
+        return dict(base, bound="alu", achieved=achieved, peak=peak, unit="TFLOP/s", frac=achieved / peak,
+                    peak_source=src + "; a multiply-add counts 2 flops")
     achieved = dom["bytes"] / secs / 1e9
     return dict(base, bound="hbm", achieved=achieved, peak=peaks["hbm_gbs"], unit="GB/s",
                 frac=achieved / peaks["hbm_gbs"], peak_source=peak_src + " copy bandwidth (MEASURED_PEAKS.json)")

@@ -13,10 +13,12 @@
 // Smoother (Section 4.2): RAS with boxes = core tiles of P nodes per axis
 // extended by `overlap`, local matrices R_i Z_k R_i^T inverted once per box
 // shape on the device (Gauss-Jordan, FP64), weights 1/multiplicity or 0/1 on
-// the core. One step z <- z + sum_i R_i^T D_i Z_i^-1 R_i (f - Z_k z) is two
-// kernels: (1) per batch of equal-shape boxes: residual on the box,
-// multiplication by the shared inverse (a small dense GEMM), results to a
-// patch-major buffer; (2) per node: weighted sum of the box results.
+// the core. One step z <- z + sum_i R_i^T D_i Z_i^-1 R_i (f - Z_k z): (1) per
+// batch of equal-shape boxes the exact local solves, results to a patch-major
+// buffer (mixed precision: a residual kernel, then products with the shared
+// inverse; FP64: ras_fix.cu, which forms the residual itself); (2) per node:
+// weighted sum of the box results. Small 2D FP64 hierarchies run all of
+// Algorithm 3 in one kernel (small_mg.cu).
 //
 // Coarsest level (Algorithm 4, k = 1): exact solve by fast diagonalisation:
 // Z_1 = (1/d) sum_i (x)_ax {K1 if ax = i else M1} with 1D Q1 matrices

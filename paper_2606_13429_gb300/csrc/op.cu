@@ -17,8 +17,8 @@
 // SM; the FP64 pipe is 82-85% busy), so its FP64 operations are what counts:
 // 46 per node in 2D (68 with a viscosity per element) against 94 of the stored
 // blocks, about 185 in 3D (310) against 890, and against 750 of the
-// matrix-free product's unfactored 27-point stencils. Measured: 100 us at
-// 1024^2, 228 us at 80^3, and with a viscosity per element 3,514 -> 1,881 us
+// matrix-free product's unfactored 27-point stencils. Measured: 107 us at
+// 1024^2, 229 us at 80^3, and with a viscosity per element 3,514 -> 1,881 us
 // at 129^3 (matrix-free).
 //
 // Mapping, 2D: a thread walks `seg` rows of one column; the row quantities
@@ -599,10 +599,12 @@ int op_time_rhs(dcg_problem* p, bool minus_div, const double* w, const double* f
 int op_product(dcg_problem* p, const OpCall& c, cudaStream_t s) {
   OpArgs a = op_args(p, c);
   if (c.slot >= 0) a.red = make_reduce(p, c.slot);
-  // algorithmic work: structural entries of the blocks (an FMA counts 2), and
-  // the vectors and 1/nu
-  const double N = (double)p->N, nn = (double)p->n_nodes, nnzb = (double)p->nnzb;
-  const double fma_blk = c.vt ? p->dim * (2 * p->dim - 1) : (p->dim == 2 ? 10 : 33);
+  // algorithmic work: FP64 instructions of the factored form per node, each
+  // counted as a multiply-add (V^T y forms the diagonal components alone),
+  // and the vectors and 1/nu
+  const double N = (double)p->N, nn = (double)p->n_nodes;
+  const double ops = (p->dim == 2 ? (a.inv_nu ? 68.0 : 46.0) : (a.inv_nu ? 310.0 : 185.0)) *
+                     (!c.vt ? 1.0 : p->dim == 2 ? 0.6 : 0.45);
   double bytes = 8.0 * ((c.x ? N : 0.0) + (c.zh ? nn : 0.0) + (c.vt ? nn : N) + (c.g ? nn : 0.0) + (c.f ? N : 0.0) +
                         (c.dvec && c.dvec != c.x ? N : 0.0) + (a.inv_nu ? nn : 0.0));
   const int prof = prof_begin(p, PC_SPMV, s);
@@ -625,7 +627,7 @@ int op_product(dcg_problem* p, const OpCall& c, cudaStream_t s) {
   }
 #undef DCG_OP
   DCG_TRY(st);
-  prof_end(p, prof, s, 2.0 * fma_blk * nnzb, bytes);
+  prof_end(p, prof, s, 2.0 * ops * nn, bytes);
   return DCG_OK;
 }
 

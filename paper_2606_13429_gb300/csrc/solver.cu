@@ -17,9 +17,10 @@
 // threshold) and x += e, at most max_restarts times.
 //
 // Per outer iteration (kernels, all FP64 except the W-cycle):
-//   g = V^T A d            (SpMV reading only the diagonal-component rows)
-//   zh = MG(g)             (Algorithm 3; one host read per W-cycle)
-//   q = A (d - V zh), d.q  (SpMV with the embed in its operand gather)
+//   t = A d, g = V^T t     (one product)
+//   zh = MG(g)             (Algorithm 3; one host read per W-cycle, or one
+//                           kernel on small 2D FP64 hierarchies)
+//   q = t - K_div V zh, d.q
 //   x += a d, r -= a q, r.r, r.q     (a from device scalars)
 //   d = r -+ b d, d.r       (b from device scalars)
 // and one host read of ||r|| for the stopping test.
