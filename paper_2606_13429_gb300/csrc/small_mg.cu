@@ -21,9 +21,9 @@
 // line solves, its rows and lines spread over the CTAs.
 //
 // Measured per inner solve (relative tolerance 1e-10, about 5 cycles), level-by-level
-// kernels in FP64 against this form: four levels, 4 x 4
-// cores: 96^2 2,782 -> 1,100 us, 32^2 2,095 -> 663 us; two levels, 8 x 8 cores,
-// 96^2 937 -> 455 us.
+// kernels with the FP64 smoother against this form: four levels, 4 x 4
+// cores: 96^2 2,782 -> 1,130 us, 32^2 2,095 -> 665 us; two levels, 8 x 8 cores,
+// 96^2 937 -> 455 us (the level-by-level kernels of today: 1,665, 1,495, 615).
 #include "ras_fix.cuh"
 
 #include <algorithm>
@@ -682,9 +682,12 @@ int sm_dispatch(const SmallState& S, const SmArgs& a, cudaStream_t s) {
 // most kSmallNodes nodes on the finest level and 80 per axis on the coarsest
 // (its dense passes grow with the cube). Per inner solve against the
 // level-by-level kernels with fixed-point smoother, us: four levels, 4 x 4
-// cores, 112^2 1,171 / 2,038, 160^2 1,427 / 2,087; two levels 64^2 323 / 446,
-// 128^2 504 / 495, 160^2 627 / 751: the gain ends a little above these sizes,
-// where a phase no longer is the latency of one round.
+// cores, 112^2 1,171 / 1,664, 160^2 1,428 / 1,733; two levels, 4 x 4 cores, 64^2
+// 324 / 428, 112^2 428 / 503, 128^2 503 / 467, 160^2 630 / 569; 8 x 8 cores, 128^2
+// 543 / 568, 160^2 675 / 679. Above these sizes a phase no longer is the
+// latency of one round; in captured solves a cycle of the level-by-level
+// kernels also pays for its loop node, so the line stays there for two
+// levels too.
 constexpr long long kSmallNodes = 26000;
 bool small_mg_supported(const dcg_problem* p) {
   const int J = (int)p->levels.size();
