@@ -679,19 +679,21 @@ int sm_dispatch(const SmallState& S, const SmArgs& a, cudaStream_t s) {
 
 // The one-kernel solve serves FP64 2D hierarchies of at least two levels whose
 // smoothed levels are box-sum levels with fixed-point local solves, with at
-// most kSmallNodes nodes on the finest level and 80 per axis on the coarsest
+// most kSmallNodes nodes on the finest level (two levels: kSmallNodes2) and 80 per axis on the coarsest
 // (its dense passes grow with the cube). Per inner solve against the
 // level-by-level kernels with fixed-point smoother, us: four levels, 4 x 4
 // cores, 112^2 1,171 / 1,664, 160^2 1,428 / 1,733; two levels, 4 x 4 cores, 64^2
 // 324 / 428, 112^2 428 / 503, 128^2 503 / 467, 160^2 630 / 569; 8 x 8 cores, 128^2
 // 543 / 568, 160^2 675 / 679. Above these sizes a phase no longer is the
-// latency of one round; in captured solves a cycle of the level-by-level
-// kernels also pays for its loop node, so the line stays there for two
-// levels too.
-constexpr long long kSmallNodes = 26000;
+// latency of one round, with two levels sooner (fewer phases per cycle, more
+// work in each): whole captured solves of two levels, 4 x 4 cores, take 8.18
+// against 6.64 ms at 128^2 and 12.22 against 10.02 at 160^2, so two levels stop
+// at kSmallNodes2.
+constexpr long long kSmallNodes = 26000, kSmallNodes2 = 13000;
 bool small_mg_supported(const dcg_problem* p) {
   const int J = (int)p->levels.size();
-  if (p->dim != 2 || p->mg.fp32 || J < 2 || J > kSmLevels || p->levels.back().nn > kSmallNodes || p->coarse.m > 80)
+  if (p->dim != 2 || p->mg.fp32 || J < 2 || J > kSmLevels || p->coarse.m > 80 ||
+      p->levels.back().nn > (J > 2 ? kSmallNodes : kSmallNodes2))
     return false;
   for (int k = 1; k < J; ++k)
     if (!p->levels[k].fdm || !p->levels[k].box) return false;

@@ -47,7 +47,8 @@ def test_matches_level_kernels(n, levels, P, o, m1, m2, weights):
     g = torch.from_numpy(inputs.rhs(11, prob.n_nodes)).cuda()
     k0 = dcg.dcg_kernel_launches()
     one = _cycles(prob, g, 2)
-    assert dcg.dcg_kernel_launches() - k0 == 1  # the one-kernel path ran
+    # the one-kernel path ran, up to its sizes: 26,000 nodes, 13,000 with two levels
+    assert (dcg.dcg_kernel_launches() - k0 == 1) == (prob.n_nodes <= (26000 if prob.levels > 2 else 13000))
     dcg.dcg_profile_enable(prob, ["coarse"])
     many = _cycles(prob, g, 2)
     dcg.dcg_profile_enable(prob, [])
