@@ -632,10 +632,15 @@ void sm_config(int ctas, int threads, size_t smem, cudaStream_t s, cudaLaunchCon
   cfg->numAttrs = 1;
 }
 
-// *fits: the device can hold one such cluster
+// shared memory a problem may plan for (227 KB less the kernel's static part)
+constexpr size_t kSmRoom = 216 * 1024;
+
+// *fits: the device can hold one such cluster. The limit on the dynamic shared
+// memory belongs to the kernel, not to a problem: every problem sets the same
+// constant, and a launch asks for what its own plan takes.
 template <int LM>
 int sm_attr(int ctas, size_t smem, bool* fits) {
-  DCG_CUDA(cudaFuncSetAttribute(k_small_mg<LM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  DCG_CUDA(cudaFuncSetAttribute(k_small_mg<LM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmRoom));
   DCG_CUDA(cudaFuncSetAttribute(k_small_mg<LM>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute at[1];
@@ -668,6 +673,7 @@ int sm_dispatch(const SmallState& S, const SmArgs& a, cudaStream_t s) {
     default: e = sm_start<16>(a, S.ctas, S.smem, s);
   }
   if (e != cudaSuccess) {
+    cudaGetLastError();  // reported here, not by the next launch check
     set_error("small multigrid solve (cluster launch)", e);
     return DCG_ERR_CUDA;
   }
@@ -765,7 +771,6 @@ int small_mg_setup(dcg_problem* p, cudaStream_t s) {
   for (int k = 1; k < J; ++k)
     work = std::max(work, sizeof(double) * p->levels[k].m *
                               (2 * ((p->levels[k - 1].m + ctas_of(k) - 1) / ctas_of(k)) + 1));
-  constexpr size_t kRoom = 216 * 1024;
   size_t used = 0, ymax = 0;
   auto take = [&](size_t bytes) {
     const size_t at = used;
@@ -809,18 +814,18 @@ int small_mg_setup(dcg_problem* p, cudaStream_t s) {
     l.o_cls = take(sizeof(int4) * L.nclass);
   }
   a.o_y = take(ymax);
-  if (used > kRoom) {  // no room for the solo levels' vectors
+  if (used > kSmRoom) {  // no room for the solo levels' vectors
     small_mg_free(p);
     return DCG_OK;
   }
   // the coarser a level, the more often a W-cycle visits it
-  a.o_S = used + sizeof(double) * m0 * m0 <= kRoom ? take(sizeof(double) * m0 * m0) : -1;
+  a.o_S = used + sizeof(double) * m0 * m0 <= kSmRoom ? take(sizeof(double) * m0 * m0) : -1;
   for (int k = 1; k < J; ++k) {
     SmLevel& l = a.lev[k];
     const int share = ctas_of(k) * nt;
     const size_t tb = sizeof(int2) * l.ntab, yb = sizeof(int4) * nt * ((l.nn + share - 1) / share);
-    l.o_tab = used + tb <= kRoom ? take(tb) : -1;
-    l.o_ysrc = used + yb <= kRoom ? take(yb) : -1;
+    l.o_tab = used + tb <= kSmRoom ? take(tb) : -1;
+    l.o_ysrc = used + yb <= kSmRoom ? take(yb) : -1;
   }
   const size_t smem = used;
   S->smem = smem;
