@@ -274,10 +274,17 @@ size_t fx_smem(const Level& L) {
   }
   return mx;
 }
+// the largest fx_smem of any level: the kernel's limit, the same for every
+// problem (a limit belongs to the kernel; a launch asks for what its level takes)
+template <int D, int LM>
+constexpr int fx_smem_max() {
+  constexpr int wb = (LM | 1) * LM * (D > 2 ? LM : 1), zn = D > 2 ? (LM + 2) * (LM + 2) * (LM + 2) : 0;
+  return 8 * fx_batch(D, LM) * (wb + zn);
+}
 
 template <int D, int LM>
-int fx_attr(const Level& L) {
-  const int smem = (int)fx_smem<D, LM>(L);
+int fx_attr() {
+  constexpr int smem = fx_smem_max<D, LM>();
   DCG_CUDA(cudaFuncSetAttribute(k_ras_fix<D, LM, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
   DCG_CUDA(cudaFuncSetAttribute(k_ras_fix<D, LM, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
   return DCG_OK;
@@ -505,14 +512,14 @@ int ras_fix_setup(dcg_problem* p, Level& L, cudaStream_t s) {
   DCG_CUDA(cudaMalloc(&L.d_fix, sizeof(int2) * tab.size()));
   DCG_CUDA(cudaMemcpyAsync(L.d_fix, tab.data(), sizeof(int2) * tab.size(), cudaMemcpyHostToDevice, s));
   DCG_CUDA(cudaStreamSynchronize(s));  // the host table goes out of scope
-  if (D == 3) return LM == 4 ? fx_attr<3, 4>(L) : fx_attr<3, 6>(L);
+  if (D == 3) return LM == 4 ? fx_attr<3, 4>() : fx_attr<3, 6>();
   switch (LM) {
-    case 4: return fx_attr<2, 4>(L);
-    case 6: return fx_attr<2, 6>(L);
-    case 8: return fx_attr<2, 8>(L);
-    case 10: return fx_attr<2, 10>(L);
-    case 12: return fx_attr<2, 12>(L);
-    default: return fx_attr<2, 16>(L);
+    case 4: return fx_attr<2, 4>();
+    case 6: return fx_attr<2, 6>();
+    case 8: return fx_attr<2, 8>();
+    case 10: return fx_attr<2, 10>();
+    case 12: return fx_attr<2, 12>();
+    default: return fx_attr<2, 16>();
   }
 }
 

@@ -57,3 +57,25 @@ def test_small_inner_solves(levels):
         for p, f in zip(ps, fs):
             st = dcg.dcg_solve(p, f, torch.zeros_like(f), tol=1e-8, max_it=2000)
             assert st["status"] == dcg.DCG_OK and st["true_relres"] <= 1e-8
+
+
+# box solves: 3D problems whose boxes are smaller than the compile-time extent
+# (6 per axis) need less shared memory, as do 2D levels with smaller boxes
+@pytest.mark.parametrize("d,first,then", [(3, (16, 4, 1), (8, 4, 1)), (3, (16, 4, 1), (12, 3, 1)),
+                                          (2, (22, 4, 1), (12, 3, 1)), (2, (46, 8, 2), (22, 7, 2))])
+def test_smoothing_steps(d, first, then):
+    ps, want = [], []
+    for n, P, o in (first, then):
+        p = dcg.dcg_assemble(d, n, 1e-4)
+        dcg.dcg_setup(p, dcg.options(max_levels=2, patch=P, overlap=o))
+        f = torch.from_numpy(inputs.rhs(33, p.n_nodes)).cuda()
+        z = torch.zeros_like(f)
+        dcg.dcg_ras_step(p, 2, f, z)
+        ps.append((p, f))
+        want.append(z)
+    for (p, f), w in zip(ps, want):  # the first again, after the second was set up
+        z = torch.zeros_like(f)
+        dcg.dcg_ras_step(p, 2, f, z)
+        assert torch.equal(z, w)
+    if d == 3:
+        _inner_solves([p for p, _ in ps], 1e-8)
