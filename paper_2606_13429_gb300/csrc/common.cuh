@@ -219,9 +219,9 @@ struct Level {
   int fdm_lmax = 0;                 // largest box extent along an axis (register bound of the kernel)
   int2* d_fix = nullptr;            // fixed-point sine matrices and line-solve factors of every class
   int fx_ntab = 0;                  // its entries
-  int fx_zb = 0, fx_gb = 0;         // bits of the quantised iterate and right-hand side / of a residual alone
-  int fx_sf = 0, fx_kout = 0;       // exponent shifts of the right-hand side and of the results
-  int2 fx_kappa{};                  // stencil factor
+  int fx_gb = 0, fx_rb = 0;         // bits of a quantised right-hand side / of a residual formed in the kernel
+  int fx_sf = 0, fx_kout = 0;       // powers of two of the right-hand side and of the results
+  int2 fx_sixth{};                  // 1/6
   double fdm_flops = 0.0;           // algorithmic flops of one fast-diagonalisation smoothing product
   void* d_inv = nullptr;            // inverses in the W-cycle precision (row-major, symmetric)
   void* d_inv_bf16 = nullptr;       // optional BF16 copy
@@ -453,7 +453,7 @@ int mg_solve(dcg_problem* p, const double* g, double* z, double tol, int nmax, i
 int ras_fix_batch(int dim, int lmax);
 int ras_fix_lm(int dim, int lmax);  // compile-time box extent that serves lmax
 int ras_fix_setup(dcg_problem* p, Level& L, cudaStream_t s);
-int ras_fix_solve(dcg_problem* p, const Level& L, bool z_zero, cudaStream_t s);
+int ras_fix_solve(dcg_problem* p, const Level& L, const double* f, const double* z, cudaStream_t s);
 // Algorithm 3 on small 2D FP64 hierarchies as one kernel (small_mg.cu)
 int small_mg_setup(dcg_problem* p, cudaStream_t s);
 void small_mg_free(dcg_problem* p);

@@ -5,9 +5,10 @@
 // 64-bit integer additions on 63. A product of a 61-bit fixed-point value
 // with a 59-bit constant takes three such multiply-adds (20.6 per clock per
 // SM measured), so a linear map of bounded values runs about ten times
-// faster in fixed point than in FP64, with a smaller rounding error: the
-// values of a block share one exponent and carry 54 to 58 bits below the
-// block's largest entry, against the 53 of an FP64 significand.
+// faster in fixed point than in FP64. The values of a block share one
+// exponent: its largest entry carries 53 to 58 bits (ras_fix.cu), smaller ones
+// fewer, against 53 for every entry in FP64, so errors are relative to the
+// block's largest entry.
 //
 // A value v (|v| < 2^60) is split as v = h 2^29 + l, |l| <= 2^28; a constant
 // c (|c| < 2) is stored as C = round(c 2^58) = c1 2^29 + c0, |c0| <= 2^28, c1
@@ -53,19 +54,13 @@ __device__ __forceinline__ unsigned fx_mag(long long bits) { return (unsigned)(b
 // implicit bit, because the field is at least 96 (a block whose largest is
 // below 2^-927 is quantised as if it were 2^-927).
 __device__ __forceinline__ int fx_block_exponent(unsigned mag) { return max((int)(mag >> 20), 96); }
-// FP64 bits to fixed point with |result| <= 2^nb: the significand moves right
-// by sh0 - (exponent field), sh0 = 63 - nb + (block exponent). fx_floor rounds
-// down (mean error -1/2 unit, the same for every entry: a stencil whose
-// coefficients sum to zero cancels it), fx_near to nearest.
+// FP64 bits to fixed point with |result| <= 2^nb, rounded to nearest: the
+// significand moves right by sh0 - (exponent field), sh0 = 63 - nb + (block
+// exponent).
 __device__ __forceinline__ long long fx_signed_significand(unsigned hi, unsigned lo) {
   const int s = (int)hi >> 31;  // one's complement: 2^-62 of the value
   const unsigned mh = __funnelshift_l(lo, (hi & 0xfffffu) | 0x100000u, 10);  // leading bit 62
   return (long long)((unsigned long long)(mh ^ (unsigned)s) << 32 | ((lo << 10) ^ (unsigned)s));
-}
-__device__ __forceinline__ long long fx_floor(long long bits, int sh0) {
-  const unsigned hi = (unsigned)(bits >> 32);
-  const int sh = min(sh0 - (int)(hi << 1 >> 21), 63);
-  return fx_signed_significand(hi, (unsigned)bits) >> sh;
 }
 __device__ __forceinline__ long long fx_near(long long bits, int sh0) {
   const unsigned hi = (unsigned)(bits >> 32);

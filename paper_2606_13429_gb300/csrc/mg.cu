@@ -16,7 +16,7 @@
 // the core. One step z <- z + sum_i R_i^T D_i Z_i^-1 R_i (f - Z_k z): (1) per
 // batch of equal-shape boxes the exact local solves, results to a patch-major
 // buffer (mixed precision: a residual kernel, then products with the shared
-// inverse; FP64: ras_fix.cu, which forms the residual itself); (2) per node:
+// inverse; FP64: ras_fix.cu, which forms the residual itself in 2D); (2) per node:
 // weighted sum of the box results. Small 2D FP64 hierarchies run all of
 // Algorithm 3 in one kernel (small_mg.cu).
 //
@@ -2152,23 +2152,25 @@ int ras_step_t(dcg_problem* p, Level& L, cudaStream_t s, bool z_zero = false) {
   const int cap = 152 * per_sm;
   ra.items_per_cta = (L.nwork + cap - 1) / cap;
   int grid = (L.nwork + ra.items_per_cta - 1) / ra.items_per_cta;
-  if constexpr (sizeof(T) == 8) {
-    if (L.fdm) {
-      // the residual of the step is formed in the kernel
-      const int prof = prof_begin(p, PC_RAS_SOLVE, s, g_capturing);
-      DCG_TRY(ras_fix_solve(p, L, z_zero, s));
-      prof_end(p, prof, s, L.fdm_flops + (z_zero ? 0.0 : 2.0 * ipow(3, D) * (double)L.nn),
-               sizeof(T) * (2.0 * (double)L.ylen + (z_zero ? 0.0 : 1.0) * L.nn), g_capturing);
-      return ras_update_t<T, D>(p, L, s);
-    }
-  }
-  // residual once per node (the first step from a zero iterate uses f itself)
+  // residual once per node (the first step from a zero iterate uses f itself,
+  // 2D FP64 box solves form it themselves)
   const T* rvec = (const T*)L.f;
-  if (!z_zero) {
+  const bool fused = D == 2 && sizeof(T) == 8 && L.fdm;
+  if (!z_zero && !fused) {
     const int prof = prof_begin(p, PC_TRANSFER, s, g_capturing);
     level_residual<T, D>(L, (const T*)L.f, (const T*)L.z, (T*)L.r, s);
     prof_end(p, prof, s, 2.0 * ipow(3, D) * (double)L.nn, sizeof(T) * 3.0 * L.nn, g_capturing);
     rvec = (const T*)L.r;
+  }
+  if constexpr (sizeof(T) == 8) {
+    if (L.fdm) {
+      const double* z = fused && !z_zero ? (const double*)L.z : nullptr;
+      const int prof = prof_begin(p, PC_RAS_SOLVE, s, g_capturing);
+      DCG_TRY(ras_fix_solve(p, L, rvec, z, s));
+      prof_end(p, prof, s, L.fdm_flops + (z ? 2.0 * ipow(3, D) * (double)L.nn : 0.0),
+               sizeof(T) * (2.0 * (double)L.ylen + (z ? 1.0 : 0.0) * L.nn), g_capturing);
+      return ras_update_t<T, D>(p, L, s);
+    }
   }
   // algorithmic work: the shared-inverse products and the data they touch
   double bytes = 0.0;

@@ -1,5 +1,5 @@
 // Exact local solves of the FP64 RAS smoother (Section 4.2) in 64-bit fixed
-// point, with the residual of the step formed in the same kernel.
+// point; in 2D with the residual of the step formed in the same kernel.
 //
 // On a level whose stencil is the Q1 Laplacian / d (checked at setup), a
 // box's local matrix R_i Z_k R_i^T is (1/d) sum_i (x)_ax {K_l if ax = i else
@@ -14,27 +14,38 @@
 // therefore goes to fixed point (fix64.cuh), where a multiply-add costs three
 // integer multiply-adds on a pipe 32 times as wide; what is left is integer
 // issue (ALU pipe 57% busy: conversions, 64-bit additions and shifts beside
-// the multiply-adds) and the load phase. Measured per launch, residual
-// included: 2D 1024^2, 8 x 8 cores with overlap 2: 85.8 + 17.4 us (solve and
-// residual kernels in FP64) -> 50.0 us, 42.1 us from a zero iterate; 3D 128^3,
-// 4^3 cores with overlap 1: 270 + 99 us -> 163.6 us, 98.1 us. Against extended
-// precision a step's error falls from 1.1e-15 to 1.7e-16 of the result (2D,
-// 12 x 12 boxes, random data) and from 4.9e-16 to 2.8e-16 (3D).
+// the multiply-adds) and the load phase. Measured per launch: 2D 1024^2, 8 x 8
+// cores with overlap 2: 85.8 + 17.4 us (solve and residual kernels in FP64)
+// -> 49.4 us, residual included, 41.8 us from a zero iterate; 3D 128^3, 4^3
+// cores with overlap 1: 270 us -> 99 us, after a residual kernel of 54 us.
 //
-// Scaling. All values of a box share one exponent, that of the largest of
-// |z| (box and its one-node halo) and |f| / hs (box), hs = 1 in 2D and the
-// power of two next below h in 3D, so that the scaled operator A / hs has
-// entries of order one whatever the level. Values are quantised to `zb` bits
-// (`gb` when the step starts from z = 0 and the residual is f itself); the
-// host chooses them from the row sums of the tables so that no intermediate
-// value can leave the range of fix64.cuh:
-//   residual growth, fold of two entries, transform |S|_inf, forward
-//   elimination, and the inverse line operators ||T_j^-1||_inf, which a
-//   transformed line j may grow by. In 2D line j is stored in units of
-//   2^K_j, K_j = ceil log2 ||T_j^-1||_inf, and the transform back multiplies
-//   by S 2^(K_j - kout); in 3D the growth is small and one K serves all.
-// A 12 x 12 box keeps 55 bits (57 from a zero iterate); an FP64 significand
-// has 53. A box with a non-finite entry returns NaN everywhere.
+// Precision. All values of a box share one exponent, so errors are relative
+// to the largest entry of the box, whose bits are (FP64: 53):
+//   right-hand side alone, step from zero and 3D: 58 (4 x 4 boxes), 57 (6 x 6),
+//   56 (8 to 12), 55 (16 x 16); 3D 56 (4^3, some mesh sizes 57), 55 (6^3, 56);
+//   residual formed here (2D): 1.6 to 0.6 bits fewer, from z and f with 58.
+// The residual is small against z near convergence, so quantising it against
+// the exponent of z would lose what FP64 keeps. In 2D it is therefore formed
+// exactly from z and f (entries within 2^5 of the largest lose nothing) and
+// gets an exponent of its own before the solve. 3D coefficients are no small
+// integers, and quantised at 56 bits a large entry over small noise left ten
+// times the error of FP64; there the residual comes from the FP64 kernel of
+// mg.cu, which also is the faster form on large grids (166 us against 99 + 54
+// at 128^3; below 48^3 a W-cycle takes up to 11% longer for the launch).
+// Error of a step against extended precision over the largest entry, FP64
+// kernels -> here: random data 1.8e-15 -> 1.8e-16 (12 x 12), 6.4e-16 -> 2.8e-16
+// (6^3); smooth z with f = Z z 1.9e-15 -> 1.7e-18, 2.1e-15 -> 1.6e-15; z falling
+// by e^1/2 per node 9.2e-17 -> 5.9e-17, 3.7e-16 -> 2.6e-16.
+//
+// Scaling. The scaled operator A / hs, hs = 1 in 2D and the power of two next
+// below h in 3D, has entries of order one whatever the level. The host
+// chooses the bits from the row sums of the tables so that no intermediate
+// value can leave the range of fix64.cuh: fold of two entries, transform
+// |S|_inf, forward elimination, and the inverse line operators ||T_j^-1||_inf,
+// which a transformed line j may grow by. In 2D line j is stored in units of
+// 2^K_j, K_j = ceil log2 ||T_j^-1||_inf, and the transform back multiplies
+// by S 2^(K_j - kout); in 3D the growth is small and one K serves all. A box
+// with a non-finite entry returns NaN everywhere.
 //
 // Mapping. A CTA takes one work item (boxes of one class). In 2D a box belongs
 // to a group of 8, 16 or 32 lanes, one per column of the box and its halo: a
@@ -43,8 +54,7 @@
 // shuffles, the y transform runs down the lane's own column, the x line solve
 // takes one row per lane, and only the two transpositions between them go
 // through shared memory; no barrier wider than a warp. In 3D a box has one
-// thread per column along z (the perimeter columns of its halo are spread
-// over the same threads) and every phase gives each thread one grid line.
+// thread per column along z and every phase gives each thread one grid line.
 // Rows are padded to an odd pitch (conflict-free 8-byte accesses).
 // A transform folds its line by the symmetry S[j][l-1-x] = (-1)^j S[j][x] (on
 // the inputs forward, on the outputs back): l^2 / 2 multiply-adds. Short
@@ -104,104 +114,38 @@ __device__ __forceinline__ void fx_boxes_2d(const FixArgs& A, const RasClass& C,
                              A.tab + C.fx_tri, [&](int q, double v) { yb[q * lx] = v; });
 }
 
-template <int LM, bool ZZERO, bool EX>
+// y = the boxes' solves of the right-hand side f
+template <int LM, bool EX>
 __device__ __forceinline__ void fx_boxes_3d(const FixArgs& A, const RasClass& C, const int2* s_tab, long long* smem, unsigned* s_e,
                                             int first, int cnt, const double* __restrict__ f,
-                                            const double* __restrict__ z, double* __restrict__ yi) {
+                                            double* __restrict__ yi) {
   constexpr int TPB = LM * LM, HP = fx_hm(LM), HM = (LM + 1) / 2, NF = LM * HP, NBK = 2 * HM * HP;
-  constexpr int NB = fx_batch(3, LM);
-  constexpr int PE = (4 * LM + 4 + TPB - 1) / TPB;  // perimeter columns per thread
   const int b = threadIdx.x / TPB, c = threadIdx.x - b * TPB;
   const int cy = c / LM, cx = c - cy * LM;
   const int lx = EX ? LM : C.len[0], ly = EX ? LM : C.len[1], lz = EX ? LM : C.len[2], m = A.m;
-  const int wp = lx | 1, hx = lx + 2, hy = ly + 2;
-  const int wb = wp * ly * lz, zn = hx * hy * (lz + 2);
-  long long* W = smem + b * wb;              // [lz][ly][wp]
-  long long* Z = smem + NB * wb + b * zn;    // [lz + 2][hy][hx]
+  const int wp = lx | 1;
+  long long* W = smem + b * (wp * ly * lz);  // [lz][ly][wp]
   const bool live = b < cnt;
   const bool own = live && cx < lx && cy < ly;
   const int4 og = live ? __ldg(A.origin + __ldg(A.class_patches + first + b)) : make_int4(0, 0, 0, 0);
   if (c == 0) s_e[b] = 0;
   __syncthreads();
   const int mm = m * m;
-  long long zv[LM + 2], fv[LM], pv[PE][LM + 2];
-  int px[PE], py[PE];
+  long long fv[LM];
   unsigned mag = 0;
-  {
-    const int base = (og.x + cx) + m * (og.y + cy) + mm * (og.z - 1);
+  const int base = (og.x + cx) + m * (og.y + cy) + mm * og.z;
 #pragma unroll
-    for (int q = 0; q < LM; ++q) {
-      fv[q] = (own && q < lz) ? __double_as_longlong(__ldg(f + base + (q + 1) * mm)) : 0;
-      const unsigned mf = fx_mag(fv[q]);
-      mag = max(mag, mf >= kFxNonFinite || mf == 0 ? mf : (unsigned)max((int)mf + (A.sc.sf << 20), 1));
-    }
-    if (!ZZERO) {
-#pragma unroll
-      for (int q = 0; q < LM + 2; ++q) {
-        const int gz = og.z - 1 + q;
-        zv[q] = (own && q <= lz + 1 && gz >= 0 && gz < m) ? __double_as_longlong(__ldg(z + base + q * mm)) : 0;
-        mag = max(mag, fx_mag(zv[q]));
-      }
-#pragma unroll
-      for (int k = 0; k < PE; ++k) {
-        // perimeter column t of the halo: the rows y = -1 and y = ly, then
-        // the sides x = -1, lx
-        const int t = c + k * TPB, u = t - 2 * hx;
-        px[k] = t < hx ? t : t < 2 * hx ? t - hx : (u & 1) ? hx - 1 : 0;
-        py[k] = t < hx ? 0 : t < 2 * hx ? hy - 1 : 1 + (u >> 1);
-        const int gx = og.x - 1 + px[k], gy = og.y - 1 + py[k];
-        const bool per = live && t < 2 * hx + 2 * ly;
-        const bool col = per && gx >= 0 && gx < m && gy >= 0 && gy < m;
-        const int pb = gx + m * gy + mm * (og.z - 1);
-#pragma unroll
-        for (int q = 0; q < LM + 2; ++q) {
-          const int gz = og.z - 1 + q;
-          pv[k][q] = (col && q <= lz + 1 && gz >= 0 && gz < m) ? __double_as_longlong(__ldg(z + pb + q * mm)) : 0;
-          mag = max(mag, fx_mag(pv[k][q]));
-        }
-        if (!per) px[k] = -1;
-      }
-    }
+  for (int q = 0; q < LM; ++q) {
+    fv[q] = (own && q < lz) ? __double_as_longlong(__ldg(f + base + q * mm)) : 0;
+    mag = max(mag, fx_mag(fv[q]));
   }
   if (live && mag) atomicMax(&s_e[b], mag);
   __syncthreads();
   mag = s_e[b];
   const int e = fx_block_exponent(mag), sh0 = 63 - A.sc.bits + e;
-  if (ZZERO) {
 #pragma unroll
-    for (int q = 0; q < LM; ++q)
-      if (own && q < lz) W[(q * ly + cy) * wp + cx] = fx_near(fv[q], sh0 - A.sc.sf);
-  } else {
-#pragma unroll
-    for (int q = 0; q < LM + 2; ++q) {
-      zv[q] = fx_floor(zv[q], sh0);
-      if (own && q <= lz + 1) Z[(q * hy + cy + 1) * hx + cx + 1] = zv[q];
-#pragma unroll
-      for (int k = 0; k < PE; ++k)
-        if (px[k] >= 0 && q <= lz + 1) Z[(q * hy + py[k]) * hx + px[k]] = fx_floor(pv[k][q], sh0);
-    }
-    __syncthreads();
-    // T = S3 + 2 S2 - 32 z (S2 the 12 edge, S3 the 8 corner neighbours; the 6
-    // face coefficients of the 3D Q1 Laplacian vanish)
-    if (own) {
-      long long Em = 0, E0 = 0, D0 = 0;
-#pragma unroll
-      for (int q = 0; q < LM + 2; ++q) {
-        const long long* p = Z + (min(q, lz + 1) * hy + cy) * hx + cx;  // planes past lz + 1 are not used
-        const long long D4 = (p[0] + p[2]) + (p[2 * hx] + p[2 * hx + 2]);
-        const long long Ep = D4 + ((p[hx] + p[hx + 2] + p[1] + p[2 * hx + 1]) << 1);
-        if (q >= 2) {
-          const long long T = Em + Ep + (D0 << 1) - (zv[q - 1] << 5);
-          FxAcc a = fx_zero();
-          fx_mac(a, fx_split(T), A.sc.kappa.x, A.sc.kappa.y);
-          if (q - 2 < lz) W[((q - 2) * ly + cy) * wp + cx] = fx_near(fv[q - 2], sh0 - A.sc.sf) + fx_value(a);
-        }
-        Em = E0;
-        E0 = Ep;
-        D0 = D4;
-      }
-    }
-  }
+  for (int q = 0; q < LM; ++q)
+    if (own && q < lz) W[(q * ly + cy) * wp + cx] = fx_near(fv[q], sh0);
   // column (cx, cy) along z; then line (cx, k = cy) along y; then line (j =
   // cx, k = cy) along x
   if (own) fx_forward<LM>(W + cy * wp + cx, ly * wp, lz, s_tab + NF + NBK);
@@ -216,7 +160,7 @@ __device__ __forceinline__ void fx_boxes_3d(const FixArgs& A, const RasClass& C,
   __syncthreads();
   if (own) {
     fx_back<LM>(W + cy * wp + cx, ly * wp, lz, s_tab + NF + NBK + NF);
-    const int e0 = e + 63 - A.sc.bits + A.sc.kout;
+    const int e0 = e + A.sc.sf + 63 - A.sc.bits + A.sc.kout;
     const bool safe = mag != 0 && mag < kFxNonFinite && e0 < 0x7ff;
     double* yb = yi + b * (lx * ly * lz) + cy * lx + cx;
     if (safe) {
@@ -251,8 +195,8 @@ __global__ void __launch_bounds__(fx_threads(D, LM), fx_blocks(D, LM))
     if (exact) fx_boxes_2d<LM, ZZERO, true>(A, C, s_tab, smem, first, cnt, f, z, yi);
     else fx_boxes_2d<LM, ZZERO, false>(A, C, s_tab, smem, first, cnt, f, z, yi);
   } else {
-    if (exact) fx_boxes_3d<LM, ZZERO, true>(A, C, s_tab, smem, s_e, first, cnt, f, z, yi);
-    else fx_boxes_3d<LM, ZZERO, false>(A, C, s_tab, smem, s_e, first, cnt, f, z, yi);
+    if (exact) fx_boxes_3d<LM, true>(A, C, s_tab, smem, s_e, first, cnt, f, yi);
+    else fx_boxes_3d<LM, false>(A, C, s_tab, smem, s_e, first, cnt, f, yi);
   }
 }
 
@@ -267,37 +211,31 @@ int2 fx_const(long long C, int shift = 0) {
 template <int D, int LM>
 size_t fx_smem(const Level& L) {
   size_t mx = 0;
-  for (const auto& c : L.classes) {
-    const size_t wb = (size_t)(c.len[0] | 1) * c.len[1] * (D > 2 ? c.len[2] : 1);
-    const size_t zn = D > 2 ? (size_t)(c.len[0] + 2) * (c.len[1] + 2) * (c.len[2] + 2) : 0;
-    mx = std::max(mx, sizeof(long long) * (size_t)c.nb * (wb + zn));
-  }
+  for (const auto& c : L.classes)
+    mx = std::max(mx, sizeof(long long) * (size_t)c.nb * (c.len[0] | 1) * c.len[1] * (D > 2 ? c.len[2] : 1));
   return mx;
 }
-// the largest fx_smem of any level: the kernel's limit, the same for every
-// problem (a limit belongs to the kernel; a launch asks for what its level takes)
+// below the 48 KB that need no limit to be raised: a limit belongs to the
+// kernel and would be shared by every problem
 template <int D, int LM>
-constexpr int fx_smem_max() {
-  constexpr int wb = (LM | 1) * LM * (D > 2 ? LM : 1), zn = D > 2 ? (LM + 2) * (LM + 2) * (LM + 2) : 0;
-  return 8 * fx_batch(D, LM) * (wb + zn);
+constexpr bool fx_smem_fits() {
+  constexpr int tab = (D - 1) * (LM + (LM + 1) / 2 * 2) * fx_hm(LM);
+  return 8 * (fx_batch(D, LM) * (LM | 1) * LM * (D > 2 ? LM : 1) + tab) + 4 * fx_batch(D, LM) <= 48 * 1024;
 }
 
+// y = solves of f - Z z on the boxes (z null: of f; 3D: z null)
 template <int D, int LM>
-int fx_attr() {
-  constexpr int smem = fx_smem_max<D, LM>();
-  DCG_CUDA(cudaFuncSetAttribute(k_ras_fix<D, LM, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-  DCG_CUDA(cudaFuncSetAttribute(k_ras_fix<D, LM, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-  return DCG_OK;
-}
-
-template <int D, int LM>
-void fx_launch(const Level& L, const FixArgs& a, bool z_zero, cudaStream_t s) {
+void fx_launch(const Level& L, const FixArgs& a, const double* f, const double* z, cudaStream_t s) {
+  static_assert(fx_smem_fits<D, LM>(), "");
   const size_t smem = fx_smem<D, LM>(L);
   constexpr int nt = fx_threads(D, LM);
-  if (z_zero)
-    k_ras_fix<D, LM, true><<<L.nwork, nt, smem, s>>>(a, (const double*)L.f, (const double*)L.z, (double*)L.y);
-  else
-    k_ras_fix<D, LM, false><<<L.nwork, nt, smem, s>>>(a, (const double*)L.f, (const double*)L.z, (double*)L.y);
+  if constexpr (D == 2) {
+    if (z) {
+      k_ras_fix<D, LM, false><<<L.nwork, nt, smem, s>>>(a, f, z, (double*)L.y);
+      return;
+    }
+  }
+  k_ras_fix<D, LM, true><<<L.nwork, nt, smem, s>>>(a, f, nullptr, (double*)L.y);
 }
 
 // compile-time extent that serves a level's largest box extent
@@ -435,8 +373,6 @@ int ras_fix_setup(dcg_problem* p, Level& L, cudaStream_t s) {
   // the lines times t1^2 bounds both).
   const double lim = 0.99 * std::ldexp(1.0, 60);
   auto bits_below = [&](double factor) { return (int)std::floor(std::log2(lim / factor)); };
-  const double kappa = D == 2 ? 1.0 / 6.0 : (double)rho / 36.0;
-  const double tz = D == 2 ? 16.0 : 64.0;  // sum of the |coefficients| of T
   const double tD = D == 2 ? t1 : t1 * t1;
   double solve = std::max(2.0, tD * grow);
   if (D == 3) solve = std::max(solve, 2.0 * t1);
@@ -465,8 +401,8 @@ int ras_fix_setup(dcg_problem* p, Level& L, cudaStream_t s) {
       K[q].push_back(k);
     }
   }
-  L.fx_zb = std::min(bits_below(tz), L.fx_gb - (int)std::ceil(std::log2(1.0 + kappa * tz)));
-  L.fx_kappa = fx_const(fx_const_bits(D == 2 ? 1.0L / 6.0L : rho / 36.0L));
+  L.fx_rb = std::min(L.fx_gb, 57);  // 6 r as an operand: at most 2^(fx_rb + 2)
+  L.fx_sixth = fx_const(fx_const_bits(1.0L / 6.0L));
 
   std::vector<int2> tab;
   for (size_t q = 0; q < L.classes.size(); ++q) {
@@ -512,19 +448,11 @@ int ras_fix_setup(dcg_problem* p, Level& L, cudaStream_t s) {
   DCG_CUDA(cudaMalloc(&L.d_fix, sizeof(int2) * tab.size()));
   DCG_CUDA(cudaMemcpyAsync(L.d_fix, tab.data(), sizeof(int2) * tab.size(), cudaMemcpyHostToDevice, s));
   DCG_CUDA(cudaStreamSynchronize(s));  // the host table goes out of scope
-  if (D == 3) return LM == 4 ? fx_attr<3, 4>() : fx_attr<3, 6>();
-  switch (LM) {
-    case 4: return fx_attr<2, 4>();
-    case 6: return fx_attr<2, 6>();
-    case 8: return fx_attr<2, 8>();
-    case 10: return fx_attr<2, 10>();
-    case 12: return fx_attr<2, 12>();
-    default: return fx_attr<2, 16>();
-  }
+  return DCG_OK;
 }
 
-// y = exact local solves of r = f - Z z on every box (z_zero: of f)
-int ras_fix_solve(dcg_problem* p, const Level& L, bool z_zero, cudaStream_t s) {
+// y = exact local solves of f - Z z on every box (z null: of f; in 3D z is null)
+int ras_fix_solve(dcg_problem* p, const Level& L, const double* f, const double* z, cudaStream_t s) {
   FixArgs a{};
   a.work = L.d_work;
   a.class_patches = L.d_class_patches;
@@ -533,19 +461,19 @@ int ras_fix_solve(dcg_problem* p, const Level& L, bool z_zero, cudaStream_t s) {
   a.item_off = L.d_item_off;
   a.tab = L.d_fix;
   a.m = L.m;
-  a.sc = FxScale{z_zero ? L.fx_gb : L.fx_zb, L.fx_sf, L.fx_kout, L.fx_kappa};
+  a.sc = ras_fix_scale(L, !z);
   const int LM = fx_lm(p->dim, L.fdm_lmax);
   if (p->dim == 3) {
-    if (LM == 4) fx_launch<3, 4>(L, a, z_zero, s);
-    else fx_launch<3, 6>(L, a, z_zero, s);
+    if (LM == 4) fx_launch<3, 4>(L, a, f, z, s);
+    else fx_launch<3, 6>(L, a, f, z, s);
   } else {
     switch (LM) {
-      case 4: fx_launch<2, 4>(L, a, z_zero, s); break;
-      case 6: fx_launch<2, 6>(L, a, z_zero, s); break;
-      case 8: fx_launch<2, 8>(L, a, z_zero, s); break;
-      case 10: fx_launch<2, 10>(L, a, z_zero, s); break;
-      case 12: fx_launch<2, 12>(L, a, z_zero, s); break;
-      default: fx_launch<2, 16>(L, a, z_zero, s);
+      case 4: fx_launch<2, 4>(L, a, f, z, s); break;
+      case 6: fx_launch<2, 6>(L, a, f, z, s); break;
+      case 8: fx_launch<2, 8>(L, a, f, z, s); break;
+      case 10: fx_launch<2, 10>(L, a, f, z, s); break;
+      case 12: fx_launch<2, 12>(L, a, f, z, s); break;
+      default: fx_launch<2, 16>(L, a, f, z, s);
     }
   }
   DCG_LAUNCH_CHECK();

@@ -13,7 +13,7 @@ constexpr int fx_group(int LM) { return LM + 2 <= 8 ? 8 : LM + 2 <= 16 ? 16 : 32
 constexpr int fx_batch(int D, int LM) { return D == 2 ? 128 / fx_group(LM) : 8; }
 constexpr int fx_threads(int D, int LM) { return D == 2 ? 128 : 8 * LM * LM; }
 // CTAs per SM the register allocation leaves room for
-constexpr int fx_blocks(int D, int LM) { return D == 2 ? (LM <= 8 ? 7 : LM <= 12 ? 6 : 4) : (LM <= 4 ? 6 : 2); }
+constexpr int fx_blocks(int D, int LM) { return D == 2 ? (LM <= 8 ? 7 : LM <= 10 ? 6 : LM <= 12 ? 5 : 4) : (LM <= 4 ? 6 : 2); }
 // pitch of a line of table constants (pairs are read as 16-byte loads)
 __host__ __device__ constexpr int fx_hm(int LM) { return ((LM + 1) / 2 + 1) / 2 * 2; }
 
@@ -165,9 +165,26 @@ __device__ __forceinline__ double fx_special(long long v, int e0, unsigned mag) 
 
 // scaling of a level's boxes
 struct FxScale {
-  int bits, sf, kout;  // bits of the quantised values; f is scaled by 2^sf; units of the results
-  int2 kappa;          // r = f 2^sf + kappa T(z), T the integer stencil sum
+  int bits, sf, kout;  // bits of the quantised residual; powers of two of the right-hand side and the results
+  int2 sixth;          // 1/6
 };
+inline FxScale ras_fix_scale(const Level& L, bool z_zero) {
+  return FxScale{z_zero ? L.fx_gb : L.fx_rb, L.fx_sf, L.fx_kout, L.fx_sixth};
+}
+
+// The residual of a 2D step is formed exactly from z and f quantised to
+// kFxZBits bits below the block's largest entry (entries within 2^5 of it lose
+// nothing): 6 r = 6 f + T(z), T = (sum of the 3 x 3 box) - 9 z, an integer of at
+// most 22 2^58 < 2^63. It then gets an exponent of its own: a shift that takes
+// its largest entry to 2^(bits + 2) at most.
+constexpr int kFxZBits = 58;
+__device__ __forceinline__ unsigned long long fx_abs1(long long v) { return (unsigned long long)(v ^ (v >> 63)); }
+__device__ __forceinline__ int fx_length(unsigned long long any) { return 64 - __clzll((long long)any); }
+__device__ __forceinline__ long long fx_res(long long v, int shift, int2 c) {
+  FxAcc a = fx_zero();
+  fx_mac(a, fx_split(shift >= 0 ? v << shift : v >> -shift), c.x, c.y);
+  return fx_value(a);
+}
 
 // Exact solve on one 2D box by a group of fx_group(LM) lanes, all lanes of the
 // warp taking part: lane `x + 1` holds column x of z (rows -1 .. ly) and f (FP64
@@ -176,7 +193,7 @@ struct FxScale {
 // EX: the box has extent LM along both axes.
 template <int LM, bool ZZERO, bool EX, typename Out>
 __device__ __forceinline__ void fx_solve_2d(const FxScale& A, int lx, int ly, bool live, const long long (&zv)[LM + 2],
-                                            const long long (&fv)[LM], long long* __restrict__ W,
+                                            long long (&fv)[LM], long long* __restrict__ W,
                                             const int2* __restrict__ tf, const int2* __restrict__ tb,
                                             const int2* __restrict__ tri, Out&& out) {
   constexpr int G = fx_group(LM);
@@ -192,28 +209,39 @@ __device__ __forceinline__ void fx_solve_2d(const FxScale& A, int lx, int ly, bo
   }
 #pragma unroll
   for (int o = G / 2; o > 0; o >>= 1) mag = max(mag, __shfl_xor_sync(0xffffffffu, mag, o, G));
-  const int e = fx_block_exponent(mag), sh0 = 63 - A.bits + e;
-  // residual r = f + kappa T(z), T = (sum of the 3 x 3 box) - 9 z
+  const int e = fx_block_exponent(mag);
+  int e0 = e + 63 + A.kout;  // of the results, less the bits of the residual
   if (ZZERO) {
+    const int sh0 = 63 - A.bits + e;
+    e0 -= A.bits;
 #pragma unroll
     for (int q = 0; q < LM; ++q)
       if (own && q < ly) W[q * wp + x] = fx_near(fv[q], sh0);
   } else {
+    const int sh0 = 63 - kFxZBits + e;
     long long s0 = 0, s1 = 0, zm = 0;
+    unsigned long long any = 0;
 #pragma unroll
     for (int q = 0; q < LM + 2; ++q) {
-      const long long zc = fx_floor(zv[q], sh0);
+      const long long zc = fx_near(zv[q], sh0);
       const long long s2 = __shfl_up_sync(0xffffffffu, zc, 1, G) + zc + __shfl_down_sync(0xffffffffu, zc, 1, G);
       if (q >= 2) {
-        const long long T = (s0 + s1 + s2) - (zm << 3) - zm;
-        FxAcc a = fx_zero();
-        fx_mac(a, fx_split(T), A.kappa.x, A.kappa.y);
-        if (own && q - 2 < ly) W[(q - 2) * wp + x] = fx_near(fv[q - 2], sh0) + fx_value(a);
+        const long long r6 = (s0 + s1 + s2) - (zm << 3) - zm + fx_near(fv[q - 2], sh0) * 6;
+        fv[q - 2] = r6;
+        if (own && q - 2 < ly) any |= fx_abs1(r6);
       }
       s0 = s1;
       s1 = s2;
       zm = zc;
     }
+    int shift = any ? fx_length(any) : 0;  // bits of the largest |6 r|
+#pragma unroll
+    for (int o = G / 2; o > 0; o >>= 1) shift = max(shift, __shfl_xor_sync(0xffffffffu, shift, o, G));
+    shift = shift ? A.bits + 2 - shift : 0;
+    e0 -= kFxZBits + shift;
+#pragma unroll
+    for (int q = 0; q < LM; ++q)
+      if (own && q < ly) W[q * wp + x] = fx_res(fv[q], shift, A.sixth);
   }
   if (own) fx_forward<LM>(W + x, wp, ly, tf);
   __syncwarp();
@@ -221,8 +249,7 @@ __device__ __forceinline__ void fx_solve_2d(const FxScale& A, int lx, int ly, bo
   __syncwarp();
   if (own) {
     fx_back<LM>(W + x, wp, ly, tb);
-    const int e0 = e + 63 - A.bits + A.kout;
-    const bool safe = mag != 0 && mag < kFxNonFinite && e0 < 0x7ff;
+    const bool safe = mag != 0 && mag < kFxNonFinite && e0 > 63 && e0 < 0x7ff;
     if (safe) {
 #pragma unroll 4
       for (int q = 0; q < ly; ++q) out(q, fx_to_double(W[q * wp + x], e0, true));

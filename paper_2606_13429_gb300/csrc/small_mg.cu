@@ -190,30 +190,43 @@ __device__ __forceinline__ void sm_box(const FxScale& sc, bool zzero, int lx, in
     }
   }
   mag = __reduce_max_sync(0xffffffffu, mag);
-  const int e = fx_block_exponent(mag), sh0 = 63 - sc.bits + e;
-  if (!zzero) {
+  const int e = fx_block_exponent(mag);
+  int e0 = e + 63 + sc.kout;
+  if (zzero) {
+    const int sh0 = 63 - sc.bits + e;
+    e0 -= sc.bits;
+#pragma unroll
+    for (int i = 0; i < NF; ++i) {
+      const int t = lane + 32 * i, q = (t * ilx) >> 16;
+      if (t < nf) W[q * wp + t - q * lx] = fx_near(fv[i], sh0);
+    }
+  } else {
+    const int sh0 = 63 - kFxZBits + e;
 #pragma unroll
     for (int i = 0; i < NZ; ++i) {
       const int t = lane + 32 * i;
-      if (t < nz) Z[t] = fx_floor(zv[i], sh0);
+      if (t < nz) Z[t] = fx_near(zv[i], sh0);
     }
     __syncwarp();
-  }
+    unsigned long long any = 0;
 #pragma unroll
-  for (int i = 0; i < NF; ++i) {
-    const int t = lane + 32 * i, q = (t * ilx) >> 16, x = t - q * lx;
-    if (t < nf) {
-      long long r = fx_near(fv[i], sh0);
-      if (!zzero) {
+    for (int i = 0; i < NF; ++i) {
+      const int t = lane + 32 * i, q = (t * ilx) >> 16, x = t - q * lx;
+      if (t < nf) {
         const long long* p = Z + q * hx + x;
         const long long c = p[hx + 1];
-        const long long T = ((p[0] + p[1] + p[2]) + (p[hx] + c + p[hx + 2]) +
-                             (p[2 * hx] + p[2 * hx + 1] + p[2 * hx + 2])) - (c << 3) - c;
-        FxAcc a = fx_zero();
-        fx_mac(a, fx_split(T), sc.kappa.x, sc.kappa.y);
-        r += fx_value(a);
+        fv[i] = ((p[0] + p[1] + p[2]) + (p[hx] + c + p[hx + 2]) + (p[2 * hx] + p[2 * hx + 1] + p[2 * hx + 2])) -
+                (c << 3) - c + fx_near(fv[i], sh0) * 6;
+        any |= fx_abs1(fv[i]);
       }
-      W[q * wp + x] = r;
+    }
+    const int len = __reduce_max_sync(0xffffffffu, any ? fx_length(any) : 0);
+    const int shift = len ? sc.bits + 2 - len : 0;
+    e0 -= kFxZBits + shift;
+#pragma unroll
+    for (int i = 0; i < NF; ++i) {
+      const int t = lane + 32 * i, q = (t * ilx) >> 16;
+      if (t < nf) W[q * wp + t - q * lx] = fx_res(fv[i], shift, sc.sixth);
     }
   }
   __syncwarp();
@@ -238,8 +251,7 @@ __device__ __forceinline__ void sm_box(const FxScale& sc, bool zzero, int lx, in
     else fx_line_solve<LM, false>(W2 + lane * wp, lx, tri + lane, ly);
   }
   __syncwarp();
-  const int e0 = e + 63 - sc.bits + sc.kout;
-  const bool safe = mag != 0 && mag < kFxNonFinite && e0 < 0x7ff;
+  const bool safe = mag != 0 && mag < kFxNonFinite && e0 > 63 && e0 < 0x7ff;
 #pragma unroll
   for (int i = 0; i < (HM * LM + 31) / 32; ++i) {
     const int t = lane + 32 * i, q = (t * ilx) >> 16, x = t - q * lx;
@@ -801,8 +813,8 @@ int small_mg_setup(dcg_problem* p, cudaStream_t s) {
     l.y = (double*)L.y;
     l.c0 = L.box_c0;
     l.c1 = L.box_c1;
-    l.sc = FxScale{L.fx_zb, L.fx_sf, L.fx_kout, L.fx_kappa};
-    l.sc0 = FxScale{L.fx_gb, L.fx_sf, L.fx_kout, L.fx_kappa};
+    l.sc = ras_fix_scale(L, false);
+    l.sc0 = ras_fix_scale(L, true);
     l.ntab = L.fx_ntab;
     l.nclass = L.nclass;
     const int each = ctas_of(k) * warps;
