@@ -49,11 +49,26 @@ __device__ __forceinline__ long long fx_value(const FxAcc& a) { return a.H + (a.
 // largest magnitude, found on the high words (IEEE order is integer order).
 constexpr unsigned kFxNonFinite = 0x7ff00000u;
 __device__ __forceinline__ unsigned fx_mag(long long bits) { return (unsigned)(bits >> 32) & 0x7fffffffu; }
-// Exponent field used for a block. Values 2^63 and more below the block's
-// largest vanish; so do zeros and subnormals, whose significand has no
-// implicit bit, because the field is at least 96 (a block whose largest is
-// below 2^-927 is quantised as if it were 2^-927).
-__device__ __forceinline__ int fx_block_exponent(unsigned mag) { return max((int)(mag >> 20), 96); }
+// A block whose largest entry lies near an end of the FP64 range (exponent
+// field below 192 or from 1856) is first scaled by 2^320 or 2^-320 and its
+// results back: entries then are normal numbers and no exponent below leaves
+// the range. In every other block zeros and subnormals, whose significand has
+// no implicit bit, lie so far below the largest entry that they vanish.
+constexpr int kFxLift = 320, kFxLowest = 192;
+__device__ __forceinline__ bool fx_odd(unsigned mag) { return mag - ((unsigned)kFxLowest << 20) >= 1664u << 20; }  // or not finite
+__device__ __forceinline__ int fx_lift(unsigned mag) {
+  return mag < (unsigned)kFxLowest << 20 ? 1 : mag >= 1856u << 20 && mag < kFxNonFinite ? -1 : 0;
+}
+__device__ __forceinline__ double fx_two320(int lift) {
+  return lift == 0 ? 1.0 : __longlong_as_double((long long)(1023 + kFxLift * lift) << 52);
+}
+__device__ __forceinline__ long long fx_scaled(long long bits, double s) {
+  return __double_as_longlong(__longlong_as_double(bits) * s);
+}
+// exponent field of a scaled block (one of subnormals counts as 2^-1022)
+__device__ __forceinline__ int fx_odd_exponent(unsigned mag, int lift) {
+  return max((int)(mag >> 20), 1) + kFxLift * lift;
+}
 // FP64 bits to fixed point with |result| <= 2^nb, rounded to nearest: the
 // significand moves right by sh0 - (exponent field), sh0 = 63 - nb + (block
 // exponent).
@@ -67,20 +82,15 @@ __device__ __forceinline__ long long fx_near(long long bits, int sh0) {
   const int sh = min(sh0 - 1 - (int)(hi << 1 >> 21), 63);
   return ((fx_signed_significand(hi, (unsigned)bits) >> sh) + 1) >> 1;
 }
-// v 2^(e0 - 1085) to FP64, rounded to nearest, |v| < 2^62; `safe` when no
-// result can leave the normal range (63 < e0 < 0x7ff), else results below it
-// are zero and above it infinite
-__device__ __forceinline__ double fx_to_double(long long v, int e0, bool safe) {
+// v 2^(e0 - 1085) to FP64, rounded to nearest, |v| < 2^62, 63 < e0 < 0x7ff (no
+// result leaves the normal range)
+__device__ __forceinline__ double fx_to_double(long long v, int e0) {
   const long long s = v >> 63;
   const unsigned long long a = (unsigned long long)((v ^ s) - s);
   const int lz = __clzll((long long)a) - 1;  // 1 .. 63
   const unsigned long long sig = ((a << lz) + 0x200) >> 10;  // 2^52 .. 2^53
-  int e = e0 - lz;  // exponent field of 2^52 <= sig < 2^53
+  const int e = e0 - lz;  // exponent field of 2^52 <= sig < 2^53
   long long bits = (long long)(((unsigned long long)(unsigned)(e - 1) << 52) + sig);
-  if (!safe) {
-    if (e <= 0) bits = 0;
-    if (e >= 0x7ff) bits = 0x7ff0000000000000ll;
-  }
   bits = a == 0 ? 0 : bits;
   return __longlong_as_double(bits | (s & (long long)0x8000000000000000ull));
 }

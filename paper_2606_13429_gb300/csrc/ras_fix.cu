@@ -110,7 +110,7 @@ __device__ __forceinline__ void fx_boxes_2d(const FixArgs& A, const RasClass& C,
       fv[q] = (own && q < ly) ? __double_as_longlong(__ldg(f + base + (q + 1) * m)) : 0;
   }
   double* yb = yi + b * (lx * ly) + x;
-  fx_solve_2d<LM, ZZERO, EX>(A.sc, lx, ly, live, zv, fv, smem + b * (ly * (lx | 1)), s_tab, s_tab + NF,
+  fx_solve_2d<LM, ZZERO, EX, true>(A.sc, lx, ly, live, zv, fv, smem + b * (ly * (lx | 1)), s_tab, s_tab + NF,
                              A.tab + C.fx_tri, [&](int q, double v) { yb[q * lx] = v; });
 }
 
@@ -142,7 +142,16 @@ __device__ __forceinline__ void fx_boxes_3d(const FixArgs& A, const RasClass& C,
   if (live && mag) atomicMax(&s_e[b], mag);
   __syncthreads();
   mag = s_e[b];
-  const int e = fx_block_exponent(mag), sh0 = 63 - A.sc.bits + e;
+  const bool odd = fx_odd(mag);
+  int e = (int)(mag >> 20);
+  if (odd) {
+    const int lift = fx_lift(mag);
+    const double up = fx_two320(lift);
+    e = fx_odd_exponent(mag, lift);
+#pragma unroll
+    for (int q = 0; q < LM; ++q) fv[q] = fx_scaled(fv[q], up);
+  }
+  const int sh0 = 63 - A.sc.bits + e;
 #pragma unroll
   for (int q = 0; q < LM; ++q)
     if (own && q < lz) W[(q * ly + cy) * wp + cx] = fx_near(fv[q], sh0);
@@ -161,11 +170,10 @@ __device__ __forceinline__ void fx_boxes_3d(const FixArgs& A, const RasClass& C,
   if (own) {
     fx_back<LM>(W + cy * wp + cx, ly * wp, lz, s_tab + NF + NBK + NF);
     const int e0 = e + A.sc.sf + 63 - A.sc.bits + A.sc.kout;
-    const bool safe = mag != 0 && mag < kFxNonFinite && e0 < 0x7ff;
     double* yb = yi + b * (lx * ly * lz) + cy * lx + cx;
-    if (safe) {
+    if (!odd) {
 #pragma unroll 2
-      for (int q = 0; q < lz; ++q) yb[q * lx * ly] = fx_to_double(W[(q * ly + cy) * wp + cx], e0, true);
+      for (int q = 0; q < lz; ++q) yb[q * lx * ly] = fx_to_double(W[(q * ly + cy) * wp + cx], e0);
     } else {
       for (int q = 0; q < lz; ++q) yb[q * lx * ly] = fx_special(W[(q * ly + cy) * wp + cx], e0, mag);
     }

@@ -157,10 +157,10 @@ __device__ __forceinline__ void fx_line_solve(long long* __restrict__ W, int n, 
   }
 }
 
-// result of a box that is all zero, has a non-finite entry, or may overflow
+__device__ __forceinline__ double fx_nan() { return __longlong_as_double(0x7ff8000000000000ll); }
+// result of a scaled box, or of one with a non-finite entry
 __device__ __forceinline__ double fx_special(long long v, int e0, unsigned mag) {
-  if (mag == 0) return 0.0;
-  return mag < kFxNonFinite ? fx_to_double(v, e0, false) : __longlong_as_double(0x7ff8000000000000ll);
+  return mag < kFxNonFinite ? fx_to_double(v, e0) * fx_two320(-fx_lift(mag)) : fx_nan();
 }
 
 // scaling of a level's boxes
@@ -190,9 +190,10 @@ __device__ __forceinline__ long long fx_res(long long v, int shift, int2 c) {
 // warp taking part: lane `x + 1` holds column x of z (rows -1 .. ly) and f (FP64
 // bits, zero outside the box or grid). W: the box's shared memory [ly][lx | 1];
 // tf, tb, tri: tables of the box's class; out(q, v) receives entry (x, q).
-// EX: the box has extent LM along both axes.
-template <int LM, bool ZZERO, bool EX, typename Out>
-__device__ __forceinline__ void fx_solve_2d(const FxScale& A, int lx, int ly, bool live, const long long (&zv)[LM + 2],
+// EX: the box has extent LM along both axes. ANY: data of any size; else at
+// least 2^-831 beside the values that count (what lies below vanishes).
+template <int LM, bool ZZERO, bool EX, bool ANY, typename Out>
+__device__ __forceinline__ void fx_solve_2d(const FxScale& A, int lx, int ly, bool live, long long (&zv)[LM + 2],
                                             long long (&fv)[LM], long long* __restrict__ W,
                                             const int2* __restrict__ tf, const int2* __restrict__ tb,
                                             const int2* __restrict__ tri, Out&& out) {
@@ -209,7 +210,19 @@ __device__ __forceinline__ void fx_solve_2d(const FxScale& A, int lx, int ly, bo
   }
 #pragma unroll
   for (int o = G / 2; o > 0; o >>= 1) mag = max(mag, __shfl_xor_sync(0xffffffffu, mag, o, G));
-  const int e = fx_block_exponent(mag);
+  const bool odd = ANY ? fx_odd(mag) : mag >= kFxNonFinite;
+  int e = ANY ? (int)(mag >> 20) : max((int)(mag >> 20), kFxLowest);
+  if (ANY && odd) {
+    const int lift = fx_lift(mag);
+    const double up = fx_two320(lift);
+    e = fx_odd_exponent(mag, lift);
+#pragma unroll
+    for (int q = 0; q < LM; ++q) fv[q] = fx_scaled(fv[q], up);
+    if (!ZZERO) {
+#pragma unroll
+      for (int q = 0; q < LM + 2; ++q) zv[q] = fx_scaled(zv[q], up);
+    }
+  }
   int e0 = e + 63 + A.kout;  // of the results, less the bits of the residual
   if (ZZERO) {
     const int sh0 = 63 - A.bits + e;
@@ -249,12 +262,11 @@ __device__ __forceinline__ void fx_solve_2d(const FxScale& A, int lx, int ly, bo
   __syncwarp();
   if (own) {
     fx_back<LM>(W + x, wp, ly, tb);
-    const bool safe = mag != 0 && mag < kFxNonFinite && e0 > 63 && e0 < 0x7ff;
-    if (safe) {
+    if (!odd) {
 #pragma unroll 4
-      for (int q = 0; q < ly; ++q) out(q, fx_to_double(W[q * wp + x], e0, true));
+      for (int q = 0; q < ly; ++q) out(q, fx_to_double(W[q * wp + x], e0));
     } else {
-      for (int q = 0; q < ly; ++q) out(q, fx_special(W[q * wp + x], e0, mag));
+      for (int q = 0; q < ly; ++q) out(q, ANY ? fx_special(W[q * wp + x], e0, mag) : fx_nan());
     }
   }
 }

@@ -190,7 +190,7 @@ __device__ __forceinline__ void sm_box(const FxScale& sc, bool zzero, int lx, in
     }
   }
   mag = __reduce_max_sync(0xffffffffu, mag);
-  const int e = fx_block_exponent(mag);
+  const int e = max((int)(mag >> 20), kFxLowest);
   int e0 = e + 63 + sc.kout;
   if (zzero) {
     const int sh0 = 63 - sc.bits + e;
@@ -251,7 +251,6 @@ __device__ __forceinline__ void sm_box(const FxScale& sc, bool zzero, int lx, in
     else fx_line_solve<LM, false>(W2 + lane * wp, lx, tri + lane, ly);
   }
   __syncwarp();
-  const bool safe = mag != 0 && mag < kFxNonFinite && e0 > 63 && e0 < 0x7ff;
 #pragma unroll
   for (int i = 0; i < (HM * LM + 31) / 32; ++i) {
     const int t = lane + 32 * i, q = (t * ilx) >> 16, x = t - q * lx;
@@ -264,9 +263,9 @@ __device__ __forceinline__ void sm_box(const FxScale& sc, bool zzero, int lx, in
         fx_mac(od, fx_split(2 * k + 1 < ly ? W2[(2 * k + 1) * wp + x] : 0), co.x, co.y);
       }
       const long long E = fx_value(ev), O = fx_value(od);
-      sm_st<SOLO>(y + q * lx + x, safe ? fx_to_double(E + O, e0, true) : fx_special(E + O, e0, mag));
+      sm_st<SOLO>(y + q * lx + x, mag < kFxNonFinite ? fx_to_double(E + O, e0) : fx_nan());
       if (q < h)
-        sm_st<SOLO>(y + (ly - 1 - q) * lx + x, safe ? fx_to_double(E - O, e0, true) : fx_special(E - O, e0, mag));
+        sm_st<SOLO>(y + (ly - 1 - q) * lx + x, mag < kFxNonFinite ? fx_to_double(E - O, e0) : fx_nan());
     }
   }
   __syncwarp();  // the next box overwrites the shared values
@@ -306,11 +305,11 @@ __device__ __forceinline__ void sm_ras(const SmLevel& L, const SmVec& V, bool zz
       long long* W = reinterpret_cast<long long*>(smem + o_work) + (warp * BPW + sub) * (LM * (LM | 1));
       auto out = [&](int q, double v) { sm_st<SOLO>(yb + q * lx, v); };
       if (zzero)
-        fx_solve_2d<LM, true, false>(sc, lx, ly, live, zv, fv, W, tab + cls.x, tab + cls.y, tab + cls.z, out);
+        fx_solve_2d<LM, true, false, false>(sc, lx, ly, live, zv, fv, W, tab + cls.x, tab + cls.y, tab + cls.z, out);
       else if (lx == LM && ly == LM)
-        fx_solve_2d<LM, false, true>(sc, LM, LM, live, zv, fv, W, tab + cls.x, tab + cls.y, tab + cls.z, out);
+        fx_solve_2d<LM, false, true, false>(sc, LM, LM, live, zv, fv, W, tab + cls.x, tab + cls.y, tab + cls.z, out);
       else
-        fx_solve_2d<LM, false, false>(sc, lx, ly, live, zv, fv, W, tab + cls.x, tab + cls.y, tab + cls.z, out);
+        fx_solve_2d<LM, false, false, false>(sc, lx, ly, live, zv, fv, W, tab + cls.x, tab + cls.y, tab + cls.z, out);
       __syncwarp();
     }
   } else
@@ -492,6 +491,35 @@ __device__ __forceinline__ void sm_run(const SmArgs& A, int op, const double* S,
   }
 }
 
+// A cycle whose residual has a norm beyond 2^+-300 starts from the residual
+// scaled to a largest entry in [1, 2), so that its boxes hold nothing near the
+// ends of the FP64 range (the box solves of a cycle leave out what lies below
+// 2^-831); the power of two that is returned (1 where it is zero or not finite)
+// comes off its correction.
+template <int NT>
+__device__ __noinline__ double sm_to_one(double* f, int nn, double* red, int rank, int ctas, double* s_red) {
+  unsigned mag = 0;
+  for (int a = rank * NT + threadIdx.x; a < nn; a += ctas * NT) mag = max(mag, fx_mag(__double_as_longlong(__ldcg(f + a))));
+  mag = __reduce_max_sync(0xffffffffu, mag);
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0) s_red[threadIdx.x >> 5] = (double)mag;
+  __syncthreads();
+  double m = 0.0;
+  for (int k = 0; k < NT / 32; ++k) m = max(m, s_red[k]);
+  sm_barrier<false>(ctas);  // the norms in `red` have been read
+  if (threadIdx.x == 0) __stcg(red + 2 * rank, m);
+  sm_barrier<false>(ctas);
+  for (int k = 0; k < ctas; ++k) m = max(m, __ldcg(red + 2 * k));
+  mag = (unsigned)m;
+  if (mag == 0 || mag >= kFxNonFinite) return 1.0;
+  // 2^1023 / 2^(field): a subnormal number for the largest field
+  const int e = 2046 - max((int)(mag >> 20), 1);
+  const double s = e > 0 ? __longlong_as_double((long long)e << 52) : __longlong_as_double(1LL << 51);
+  for (int a = rank * NT + threadIdx.x; a < nn; a += ctas * NT) __stcg(f + a, __ldcg(f + a) * s);
+  sm_barrier<false>(ctas);
+  return s;
+}
+
 template <int LM>
 __global__ void __launch_bounds__(sm_threads(LM), 1) k_small_mg(const __grid_constant__ SmArgs A) {
   constexpr int NT = sm_threads(LM);
@@ -547,6 +575,8 @@ __global__ void __launch_bounds__(sm_threads(LM), 1) k_small_mg(const __grid_con
       if (!(gn > 0.0) || !(rn / gn > tol)) break;
     }
     if (n >= A.nmax) break;
+    double scale = 1.0;
+    if (!(rr >= 0x1p-600 && rr <= 0x1p600)) scale = sm_to_one<NT>(T.f, T.nn, A.red, rank, ctas, s_red);
     for (int k = 0; k < A.nops; ++k) {
       const int op = __ldg(A.ops + k);
       if ((op & 255) != SM_SOLO) {
@@ -566,7 +596,7 @@ __global__ void __launch_bounds__(sm_threads(LM), 1) k_small_mg(const __grid_con
       sm_barrier<false>(ctas);
     }
     for (int a = rank * NT + threadIdx.x; a < T.nn; a += ctas * NT)
-      __stcg(A.z + a, __ldcg(A.z + a) + __ldcg(T.z + a));
+      __stcg(A.z + a, __ldcg(A.z + a) + (scale == 1.0 ? __ldcg(T.z + a) : __ldcg(T.z + a) / scale));
     sm_barrier<false>(ctas);
     ++n;
   }
