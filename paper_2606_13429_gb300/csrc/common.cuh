@@ -458,8 +458,8 @@ int ras_fix_solve(dcg_problem* p, const Level& L, const double* f, const double*
 int small_mg_setup(dcg_problem* p, cudaStream_t s);
 void small_mg_free(dcg_problem* p);
 inline bool small_mg_ready(const dcg_problem* p) { return p->mg.small != nullptr && p->prof.mask == 0; }
-int small_mg_launch(dcg_problem* p, const double* g, double* z, double tol, int nmax, const double* tol_dev, int* total,
-                    int* iter, const int* in_iter, cudaStream_t s);
+int small_mg_launch(dcg_problem* p, const double* g, double* z, bool fixed, double tol, int nmax, const double* tol_dev,
+                    int* total, int* iter, const int* in_iter, cudaStream_t s);
 int small_mg_cycles_done(dcg_problem* p, int* ncyc, cudaStream_t s);
 std::vector<int> level_sizes(int n, int max_levels);  // mesh sizes n_J, n_J/2, ... (finest first)
 int mg_ras_step_hook(dcg_problem* p, int level, const double* f, double* z, cudaStream_t s);

@@ -263,7 +263,7 @@ struct Builder {
     DCG_LAUNCH_CHECK();
     DCG_TRY(zero(z, p->n_nodes, s));
     if (small_mg_ready(p))
-      return small_mg_launch(p, g, z, 0.0, p->opts.inner_nmax, &S->mg_tol, &S->total_cycles, &S->iter_cycles,
+      return small_mg_launch(p, g, z, false, 0.0, p->opts.inner_nmax, &S->mg_tol, &S->total_cycles, &S->iter_cycles,
                              &S->mg_in_iter, s);
     DCG_TRY(mg_graph_residual(p, g, z, true, s));
     cudaGraphConditionalHandle h = 0;

@@ -2628,7 +2628,7 @@ int exact_solve(dcg_problem* p, const double* g, double* z, cudaStream_t s) {
 int mg_cycles(dcg_problem* p, const double* g, double* z, int ncycles, cudaStream_t s) {
   if (p->levels.empty()) return DCG_ERR_STATE;
   if (exact_mode(p)) return exact_solve(p, g, z, s);
-  if (small_mg_ready(p)) return small_mg_launch(p, g, z, -1.0, ncycles, nullptr, nullptr, nullptr, nullptr, s);
+  if (small_mg_ready(p)) return small_mg_launch(p, g, z, true, 0.0, ncycles, nullptr, nullptr, nullptr, nullptr, s);
   const bool fp32 = p->mg.fp32;
   for (int c = 0; c < ncycles; ++c) {
     DCG_TRY(fp32 ? inner_residual<float>(p, g, z, s) : inner_residual<double>(p, g, z, s));
@@ -2648,7 +2648,7 @@ int mg_solve(dcg_problem* p, const double* g, double* z, double tol, int nmax, i
   *ncyc = 0;
   if (exact_mode(p)) return exact_solve(p, g, z, s);
   if (small_mg_ready(p)) {
-    DCG_TRY(small_mg_launch(p, g, z, tol, nmax, nullptr, nullptr, nullptr, nullptr, s));
+    DCG_TRY(small_mg_launch(p, g, z, false, tol, nmax, nullptr, nullptr, nullptr, nullptr, s));
     return small_mg_cycles_done(p, ncyc, s);
   }
   const bool fp32 = p->mg.fp32;

@@ -77,14 +77,14 @@ struct SmArgs {
   // per call
   const double* g;
   double* z;
-  double tol;              // relative tolerance; < 0: exactly nmax cycles
+  int fixed;               // exactly nmax cycles, no test
+  double tol;              // relative tolerance
   const double* tol_dev;   // read instead of tol when set
   int nmax;
   int* ncyc;               // cycles done
   int *total, *iter;       // counters to add them to (may be null)
   const int* in_iter;      // add to `iter` too when set and nonzero
   double* red;             // [2 * kSmCtas]
-  double* norms;           // out: ||r||^2, ||g||^2
 };
 
 // Phases run on the cluster's CTAs (SOLO = false: vectors in global memory,
@@ -564,12 +564,8 @@ __global__ void __launch_bounds__(sm_threads(LM), 1) k_small_mg(const __grid_con
       rr += __ldcg(A.red + 2 * k);
       gg += __ldcg(A.red + 2 * k + 1);
     }
-    if (rank == 0 && threadIdx.x == 0) {
-      A.norms[0] = rr;
-      A.norms[1] = gg;
-    }
     // Algorithm 3's test, the same decision in every thread
-    if (tol >= 0.0) {
+    if (!A.fixed) {
       const double rn = sqrt(rr);
       if (n == 0) gn = sqrt(gg);
       if (!(gn > 0.0) || !(rn / gn > tol)) break;
@@ -635,7 +631,7 @@ struct SmallState {
   int* ops = nullptr;
   int* boxes = nullptr;    // [2] per box of every smoothed level
   double* tri = nullptr;   // [2 m^2 + m]
-  double* red = nullptr;   // [2 * kSmCtas + 2]
+  double* red = nullptr;   // [2 * kSmCtas]
   int* ncyc = nullptr;
 };
 
@@ -881,7 +877,7 @@ int small_mg_setup(dcg_problem* p, cudaStream_t s) {
   a.nsolo = (int)ops.size() - a.nops;
   DCG_CUDA(cudaMalloc(&S->ops, sizeof(int) * ops.size()));
   DCG_CUDA(cudaMalloc(&S->tri, sizeof(double) * (2 * (size_t)m0 * m0 + m0)));
-  DCG_CUDA(cudaMalloc(&S->red, sizeof(double) * (2 * kSmCtas + 2)));
+  DCG_CUDA(cudaMalloc(&S->red, sizeof(double) * 2 * kSmCtas));
   DCG_CUDA(cudaMalloc(&S->ncyc, sizeof(int)));
   DCG_CUDA(cudaMemcpyAsync(S->ops, ops.data(), sizeof(int) * ops.size(), cudaMemcpyHostToDevice, s));
   k_small_tri<<<(m0 + 63) / 64, 64, 0, s>>>(m0, S->tri, S->tri + (size_t)m0 * m0, S->tri + 2 * (size_t)m0 * m0);
@@ -893,7 +889,6 @@ int small_mg_setup(dcg_problem* p, cudaStream_t s) {
   a.tw = S->tri + (size_t)m0 * m0;
   a.te = S->tri + 2 * (size_t)m0 * m0;
   a.red = S->red;
-  a.norms = S->red + 2 * kSmCtas;
   a.ncyc = S->ncyc;
   bool fits = false;
   switch (S->lm) {
@@ -909,14 +904,15 @@ int small_mg_setup(dcg_problem* p, cudaStream_t s) {
 }
 
 // Algorithm 3 on g from the iterate z: until ||g - Z z|| <= tol ||g|| or nmax
-// cycles (tol < 0: exactly nmax); the cycle count is left on the device.
+// cycles (fixed: exactly nmax); the cycle count is left on the device.
 // tol_dev, total, iter, in_iter: device operands of the captured solve.
-int small_mg_launch(dcg_problem* p, const double* g, double* z, double tol, int nmax, const double* tol_dev, int* total,
-                    int* iter, const int* in_iter, cudaStream_t s) {
+int small_mg_launch(dcg_problem* p, const double* g, double* z, bool fixed, double tol, int nmax, const double* tol_dev,
+                    int* total, int* iter, const int* in_iter, cudaStream_t s) {
   SmallState* S = static_cast<SmallState*>(p->mg.small);
   SmArgs a = S->args;
   a.g = g;
   a.z = z;
+  a.fixed = fixed;
   a.tol = tol;
   a.tol_dev = tol_dev;
   a.nmax = nmax;
