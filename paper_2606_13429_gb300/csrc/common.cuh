@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <atomic>
 #include <cstdint>
+#include <memory>
 #include <string>
 #include <vector>
 
@@ -211,6 +212,7 @@ struct Level {
   int* d_ysrc = nullptr;            // [nn * 2^d] index in y of each node's box results, -1 = none
   void* r = nullptr;                // residual f - Z z (cycle precision)
   int nwork = 0;
+  std::vector<int> item_count;      // boxes of each work item (host copy)
   long long ylen = 0;
   long long ras_np2 = 0;            // sum over boxes of np^2 (FMAs of one smoothing product)
   long long gmax = 0;               // max over classes of np * nb (residual tile elements)
@@ -452,7 +454,9 @@ int mg_solve(dcg_problem* p, const double* g, double* z, double tol, int nmax, i
 // FP64 smoother's local solves in 64-bit fixed point (ras_fix.cu)
 int ras_fix_batch(int dim, int lmax);
 int ras_fix_lm(int dim, int lmax);  // compile-time box extent that serves lmax
-int ras_fix_setup(dcg_problem* p, Level& L, cudaStream_t s);
+struct FixTables;  // constants the levels of one hierarchy share while it is set up
+std::shared_ptr<FixTables> ras_fix_tables();
+int ras_fix_setup(dcg_problem* p, Level& L, FixTables& shared, cudaStream_t s);
 int ras_fix_solve(dcg_problem* p, const Level& L, const double* f, const double* z, cudaStream_t s);
 // Algorithm 3 on small 2D FP64 hierarchies as one kernel (small_mg.cu)
 int small_mg_setup(dcg_problem* p, cudaStream_t s);

@@ -1810,7 +1810,7 @@ void free_level(Level& L) {
 
 // lmax_all: the largest box extent of any level (the levels share the
 // compile-time extent of their fixed-point tables)
-int setup_ras(dcg_problem* p, Level& L, bool fp32, int lmax_all, cudaStream_t s) {
+int setup_ras(dcg_problem* p, Level& L, bool fp32, int lmax_all, FixTables& fix, cudaStream_t s) {
   const int D = p->dim;
   const dcg_options& o = p->opts;
   L.tc = fp32 && o.ras_inverse == DCG_INV_BF16;  // BF16 inverses on the tensor cores
@@ -1891,6 +1891,8 @@ int setup_ras(dcg_problem* p, Level& L, bool fp32, int lmax_all, cudaStream_t s)
     }
   }
   L.nwork = (int)work.size() / 3;
+  L.item_count.clear();
+  for (int w = 0; w < L.nwork; ++w) L.item_count.push_back(work[3 * (size_t)w + 2]);
   // box origins, packed local coordinates per class, per-coordinate box table
   std::vector<int4> origin(L.npatch);
   std::vector<int2> core(L.npatch);
@@ -1990,7 +1992,7 @@ int setup_ras(dcg_problem* p, Level& L, bool fp32, int lmax_all, cudaStream_t s)
   const size_t tsz = fp32 ? sizeof(float) : sizeof(double);
   // fast-diagonalisation tables
   if (L.fdm) {
-    DCG_TRY(ras_fix_setup(p, L, s));
+    DCG_TRY(ras_fix_setup(p, L, fix, s));
     DCG_CUDA(cudaMemcpyAsync(L.d_classes, L.classes.data(), sizeof(RasClass) * L.nclass, cudaMemcpyHostToDevice, s));
     // algorithmic flops of one smoothing product (an FMA counts 2): folded
     // transforms along every axis but the last, forward and back, and the
@@ -2452,6 +2454,7 @@ int mg_setup(dcg_problem* p, cudaStream_t s) {
   // --- buffers and RAS
   const size_t tsz = fp32 ? sizeof(float) : sizeof(double);
   p->mg.fp32 = fp32;
+  const std::shared_ptr<FixTables> fix = ras_fix_tables();
   int lmax_all = 1;
   for (int k = 1; k < J; ++k) lmax_all = std::max(lmax_all, std::min(p->levels[k].m, o.patch + 2 * o.overlap));
   for (int k = 0; k < J; ++k) {
@@ -2459,7 +2462,7 @@ int mg_setup(dcg_problem* p, cudaStream_t s) {
     DCG_CUDA(cudaMalloc(&L.f, tsz * L.nn));
     DCG_CUDA(cudaMalloc(&L.z, tsz * L.nn));
     DCG_CUDA(cudaMemsetAsync(L.z, 0, tsz * L.nn, s));
-    if (k >= 1) DCG_TRY(setup_ras(p, L, fp32, lmax_all, s));
+    if (k >= 1) DCG_TRY(setup_ras(p, L, fp32, lmax_all, *fix, s));
   }
   // --- coarsest solver
   {
@@ -2548,18 +2551,21 @@ int mg_setup(dcg_problem* p, cudaStream_t s) {
   DCG_TRY(set_ras_smem(k_ras_solve<double, 3, true>));
   DCG_TRY(set_ras_smem(k_ras_solve<double, 2, false>));
   DCG_TRY(set_ras_smem(k_ras_solve<double, 3, false>));
+  if (!exact_mode(p)) DCG_TRY(small_mg_setup(p, s));
   DCG_CUDA(cudaStreamSynchronize(s));
   if (p->matrix_free) DCG_TRY(mf_check_stencil(p, s));
-  if (!exact_mode(p)) {
-    DCG_TRY(small_mg_setup(p, s));
-    DCG_TRY(build_wcycle_graph(p));
-  }
+  // (the one-kernel solve needs no W-cycle graph; kernel-class timing does)
+  if (!exact_mode(p) && !small_mg_ready(p)) DCG_TRY(build_wcycle_graph(p));
   return DCG_OK;
 }
 
 int mg_rebuild_graph(dcg_problem* p) {
   if (p->levels.empty() || exact_mode(p)) return DCG_OK;
-  return build_wcycle_graph(p);
+  if (!small_mg_ready(p)) return build_wcycle_graph(p);
+  if (p->mg.wexec) cudaGraphExecDestroy(p->mg.wexec);
+  p->mg.wexec = nullptr;
+  prof_clear_graph(p);
+  return DCG_OK;
 }
 
 int mg_inner_apply(dcg_problem* p, const double* z, double* y, cudaStream_t s) {

@@ -66,6 +66,7 @@
 #include <algorithm>
 #include <cmath>
 #include <map>
+#include <memory>
 #include <utility>
 
 namespace dcg {
@@ -208,7 +209,57 @@ __global__ void __launch_bounds__(fx_threads(D, LM), fx_blocks(D, LM))
   }
 }
 
-long long fx_const_bits(long double c) { return (long long)llroundl(c * 288230376151711744.0L); }  // 2^58
+// Double-double numbers (sums of two doubles, about 104 bits, by Dekker's and
+// Knuth's error-free sum and product). The tables are formed in them because
+// long double is software on Arm (3D, 4^3 cores: 645 us per level with it, a
+// third of the set-up at 16^3).
+struct Dd {
+  double h, l;
+};
+// (a call of its own: its operands have to be rounded before they are added,
+// and compilers for Arm fuse an inlined product into the addition)
+__attribute__((noinline)) Dd dd_sum(double a, double b) {
+  const double s = a + b, t = s - a;
+  return Dd{s, (a - (s - t)) + (b - t)};
+}
+Dd operator+(Dd a, Dd b) {
+  const Dd s = dd_sum(a.h, b.h);
+  return dd_sum(s.h, s.l + (a.l + b.l));
+}
+Dd operator-(Dd a) { return Dd{-a.h, -a.l}; }
+Dd operator-(Dd a, Dd b) { return a + -b; }
+Dd operator*(Dd a, Dd b) {
+  const double p = a.h * b.h;
+  return dd_sum(p, std::fma(a.h, b.h, -p) + std::fma(a.h, b.l, a.l * b.h));
+}
+Dd dd_inverse(Dd a) {
+  const double q = 1.0 / a.h;
+  const Dd r = Dd{1.0, 0.0} - a * Dd{q, 0.0};
+  return dd_sum(q, q * (r.h + r.l));
+}
+Dd operator/(Dd a, double b) { return a * dd_inverse(Dd{b, 0.0}); }
+Dd dd_root(double x) {  // of x > 0: one Newton step
+  const double y = std::sqrt(x);
+  return dd_sum(y, std::fma(-y, y, x) / (2.0 * y));
+}
+// sine and cosine of 0 < x <= pi / 4 by their series
+void dd_sincos(Dd x, Dd* sn, Dd* cs) {
+  const Dd x2 = -(x * x);
+  Dd t{1.0, 0.0}, s{0.0, 0.0}, c{0.0, 0.0};
+  for (int k = 1; std::fabs(t.h) > 1e-34; ++k) {  // t = (-1)^(k-1) x^(2k-2) / (2k - 2)!
+    c = c + t;
+    const Dd u = t / (2.0 * k - 1.0);
+    s = s + u;
+    t = u * x2 / (2.0 * k);
+  }
+  *sn = s * x;
+  *cs = c;
+}
+// round(c 2^58)
+long long fx_const_bits(Dd c) {
+  const double v = std::nearbyint(c.h * 0x1p58);
+  return (long long)v + (long long)std::nearbyint(std::fma(c.h, 0x1p58, -v) + c.l * 0x1p58);
+}
 // the constant C 2^-58 2^shift as the pair fx_mac takes
 int2 fx_const(long long C, int shift = 0) {
   const long long v = shift >= 0 ? C << shift : (C + (1LL << (-shift - 1))) >> -shift;
@@ -257,121 +308,154 @@ int fx_lm(int dim, int lmax) {
 int ras_fix_lm(int dim, int lmax) { return fx_lm(dim, lmax); }
 int ras_fix_batch(int dim, int lmax) { return fx_batch(dim, fx_lm(dim, lmax)); }
 
+// What the levels of one hierarchy share while it is set up
+struct FixExtent {
+  std::vector<Dd> kap, mu;     // 1D eigenvalues at h = 1
+  std::vector<long long> S;    // sine matrix
+  double row = 0.0, mx = 0.0;  // largest absolute row sum and entry of S
+};
+// Line systems along x after the transforms along y (j) and z (k), system
+// j + ly k: the tridiagonal Toeplitz part of A', the same for every extent
+// along x (a shorter line takes the first of `rows` factors). Per row i: -l_i,
+// winv_i, -b winv_i; and for lines of `rows` the reciprocal pivot of the row
+// that meets an equal elimination of half of them from the other end.
+struct FixLines {
+  std::vector<long long> l, w, bw, meet;  // meet: one per system
+  std::vector<double> ld, wd, b;          // |l_i|, winv_i; |b| per system
+};
+struct FixTables {
+  double rho = 0.0;  // the lines' scale
+  std::map<int, FixExtent> ext;
+  std::map<std::pair<int, int>, FixLines> lines;
+};
+std::shared_ptr<FixTables> ras_fix_tables() { return std::make_shared<FixTables>(); }
+
+namespace {
+// sines and cosines of pi k / (2 N), N = l + 1, by the rotation from k to k + 1
+FixExtent fix_extent(int l) {
+  const int N = l + 1;
+  const Dd pi{3.141592653589793116, 1.2246467991473531772e-16}, nrm = dd_inverse(dd_root(N / 2.0));
+  std::vector<Dd> q(N + 1, Dd{0.0, 0.0});
+  Dd s1, c1, c{1.0, 0.0};
+  dd_sincos(pi / (2.0 * N), &s1, &c1);
+  for (int k = 0; k < N; ++k) {
+    q[k + 1] = q[k] * c1 + c * s1;
+    c = c * c1 - q[k] * s1;
+  }
+  FixExtent e;
+  std::vector<long long> sn(N, 0);
+  for (int j = 1; j < N; ++j) sn[j] = fx_const_bits(nrm * q[2 * j <= N ? 2 * j : 2 * N - 2 * j]);
+  e.S.resize((size_t)l * l);
+  for (int j = 0; j < l; ++j) {
+    double t = 0.0;
+    for (int x = 0; x < l; ++x) {
+      const int a = ((j + 1) * (x + 1)) % (2 * N);
+      const long long v = a <= l ? sn[a] : a == N ? 0 : -sn[a - N];
+      e.S[(size_t)j * l + x] = v;
+      const double av = std::fabs((double)v * 0x1p-58);
+      t += av;
+      e.mx = std::max(e.mx, av);
+    }
+    e.row = std::max(e.row, t);
+    const int k = 2 * (j + 1);
+    const Dd cs = k <= N ? q[N - k] : -q[k - N], d = Dd{1.0, 0.0} - cs;
+    e.kap.push_back(d + d);
+    e.mu.push_back((Dd{2.0, 0.0} + cs) / 3.0);
+  }
+  return e;
+}
+
+FixLines fix_lines(int D, const FixExtent& ey, const FixExtent& ez, int ly, int lz, int rows, Dd rho) {
+  FixLines v;
+  const int nsys = ly * lz;
+  v.l.resize((size_t)nsys * rows);
+  v.w = v.bw = v.l;
+  v.ld.resize((size_t)nsys * rows);
+  v.wd = v.ld;
+  v.meet.resize(nsys);
+  v.b.resize(nsys);
+  for (int sys = 0; sys < nsys; ++sys) {
+    const int j = sys % ly, k = sys / ly;
+    const Dd cm = D == 2 ? ey.kap[j] / 2.0 : (ey.kap[j] * ez.mu[k] + ey.mu[j] * ez.kap[k]) / 3.0;
+    const Dd ck = D == 2 ? ey.mu[j] / 2.0 : ey.mu[j] * ez.mu[k] / 3.0;
+    const Dd a = rho * (cm / 1.5 + ck + ck), bb = rho * (cm / 6.0 - ck);
+    v.b[sys] = std::fabs(bb.h);
+    Dd wi{0.0, 0.0};  // reciprocal pivot
+    for (int i = 0; i < rows; ++i) {
+      const size_t at = (size_t)sys * rows + i;
+      const Dd li = bb * wi, w = a - li * bb;
+      wi = dd_inverse(w);
+      const Dd bw = bb * wi;
+      v.l[at] = fx_const_bits(-li);
+      v.w[at] = fx_const_bits(wi);
+      v.bw[at] = fx_const_bits(-bw);
+      v.ld[at] = std::fabs(li.h);
+      v.wd[at] = wi.h;
+      if (i == rows / 2 - 1) v.meet[sys] = fx_const_bits(dd_inverse(w - bb * bw));
+    }
+  }
+  return v;
+}
+
+// ||T^-1||_inf of a line of n rows: |T^-1| is the inverse with off-diagonals
+// -|b|, and its row sums solve that system for a right-hand side of ones;
+// *grow: bound of the forward sweep for |g| <= 1
+double fix_line_norm(const double* ld, const double* wd, double b, int n, double* grow) {
+  double v[16], u = 0.0, norm = 0.0;
+  for (int i = 0; i < n; ++i) {
+    v[i] = u = 1.0 + ld[i] * u;
+    *grow = std::max(*grow, u);
+  }
+  for (int i = n - 1; i >= 0; --i) {
+    v[i] = (v[i] + (i + 1 < n ? b * v[i + 1] : 0.0)) * wd[i];
+    norm = std::max(norm, v[i]);
+  }
+  return norm;
+}
+}  // namespace
+
 // Tables of a level's box classes and its quantisation (see the file header).
-int ras_fix_setup(dcg_problem* p, Level& L, cudaStream_t s) {
-  typedef long double ld;
+// `shared`: what the hierarchy's other levels have formed already.
+int ras_fix_setup(dcg_problem* p, Level& L, FixTables& shared, cudaStream_t s) {
   const int D = p->dim, LM = fx_lm(D, L.fdm_lmax), HM = (LM + 1) / 2, HP = fx_hm(LM);
-  const ld pi = acosl(-1.0L);
   // A' = A / hs = rho * (the operator at h = 1)
-  ld rho = 1.0L;
+  Dd rho{1.0, 0.0};
   L.fx_sf = 0;
   if (D == 3) {
     int e = 0;
-    const ld fr = frexpl(1.0L / L.n, &e);  // h = fr 2^e, fr in [0.5, 1)
-    rho = 2.0L * fr;
+    std::frexp(1.0 / L.n, &e);  // h = fr 2^e, fr in [0.5, 1)
+    const double two = std::ldexp(1.0, 1 - e);
+    rho = dd_inverse(Dd{(double)L.n, 0.0});
+    rho = Dd{rho.h * two, rho.l * two};
     L.fx_sf = -(e - 1);
   }
-  // Constants are formed in extended precision, once per extent and per pair
-  // of extents along y and z (extended precision is software on Arm), and
-  // kept as integers C = round(c 2^58); the bounds need doubles only.
-  struct Ext {
-    std::vector<ld> kap, mu;    // 1D eigenvalues at h = 1
-    std::vector<long long> S;   // sine matrix
-    double row = 0.0, mx = 0.0; // largest absolute row sum and entry of S
-  };
-  std::map<int, Ext> ext;
-  int nmax = 0;
-  for (const auto& c : L.classes) {
-    nmax = std::max(nmax, c.len[0]);
-    for (int k = 0; k < D; ++k) {
-      const int l = c.len[k];
-      if (ext.count(l)) continue;
-      Ext& e = ext[l];
-      const ld nrm = sqrtl(2.0L / (l + 1));
-      std::vector<long long> sn(l + 1);
-      for (int j = 0; j <= l; ++j) sn[j] = j == 0 ? 0 : fx_const_bits(nrm * sinl(pi * j / (l + 1)));
-      for (int j = 0; j < l; ++j) {
-        double t = 0.0;
-        for (int x = 0; x < l; ++x) {
-          const int a = ((j + 1) * (x + 1)) % (2 * (l + 1));
-          e.S.push_back(a <= l ? sn[a] : a == l + 1 ? 0 : -sn[a - l - 1]);
-          const double v = std::fabs(std::ldexp((double)e.S.back(), -58));
-          t += v;
-          e.mx = std::max(e.mx, v);
-        }
-        e.row = std::max(e.row, t);
-        const ld cs = cosl(pi * (j + 1) / (l + 1));
-        e.kap.push_back(2.0L * (1.0L - cs));
-        e.mu.push_back((2.0L + cs) / 3.0L);
-      }
-    }
+  // Constants are formed once per extent and per pair of extents along y and
+  // z, and kept as integers C = round(c 2^58); the bounds need doubles only.
+  if (shared.rho != rho.h) {
+    shared.lines.clear();
+    shared.rho = rho.h;
   }
-  // Line systems along x after the transforms along y (j) and z (k): the
-  // tridiagonal Toeplitz part of A', the same for every extent along x (a
-  // shorter line takes the first factors). Per row i: -l_i, winv_i,
-  // -b winv_i, and the reciprocal pivot of the row that meets an equal
-  // elimination of i + 1 rows from the other end.
-  struct Line {
-    std::vector<long long> l, w, bw, meet;
-    std::vector<double> ld_, wd;  // |l_i| and winv_i
-    double b;
+  std::map<int, FixExtent>& ext = shared.ext;
+  auto lines_of = [&](const RasClass& c) -> const FixLines& {
+    return shared.lines.at(std::pair<int, int>(c.len[1], D == 2 ? 1 : c.len[2]));
   };
-  std::map<std::pair<int, int>, std::vector<Line>> lines;
   for (const auto& c : L.classes) {
+    for (int k = 0; k < D; ++k)
+      if (!ext.count(c.len[k])) ext.emplace(c.len[k], fix_extent(c.len[k]));
     const std::pair<int, int> key(c.len[1], D == 2 ? 1 : c.len[2]);
-    if (lines.count(key)) continue;
-    std::vector<Line>& v = lines[key];
-    const Ext &ey = ext[c.len[1]], &ez = ext[c.len[D - 1]];
-    for (int sys = 0; sys < key.first * key.second; ++sys) {
-      const int j = sys % key.first, k = sys / key.first;
-      const ld cm = D == 2 ? ey.kap[j] / 2.0L : (ey.kap[j] * ez.mu[k] + ey.mu[j] * ez.kap[k]) / 3.0L;
-      const ld ck = D == 2 ? ey.mu[j] / 2.0L : ey.mu[j] * ez.mu[k] / 3.0L;
-      const ld a = rho * (cm * (4.0L / 6.0L) + ck * 2.0L), bb = rho * (cm / 6.0L - ck);
-      Line r;
-      r.b = std::fabs((double)bb);
-      ld wi = 0.0L;  // reciprocal pivot
-      for (int i = 0; i < nmax; ++i) {
-        const ld li = bb * wi, w = a - li * bb;
-        wi = 1.0L / w;
-        const ld bw = bb * wi;
-        r.l.push_back(fx_const_bits(-li));
-        r.w.push_back(fx_const_bits(wi));
-        r.bw.push_back(fx_const_bits(-bw));
-        r.meet.push_back(fx_const_bits(1.0L / (w - bb * bw)));
-        r.ld_.push_back(std::fabs((double)li));
-        r.wd.push_back((double)wi);
-      }
-      v.push_back(r);
-    }
+    if (!shared.lines.count(key))
+      shared.lines.emplace(key, fix_lines(D, ext.at(c.len[1]), ext.at(c.len[D - 1]), key.first, key.second, LM, rho));
   }
-  auto lines_of = [&](const RasClass& c) -> const std::vector<Line>& {
-    return lines.at(std::pair<int, int>(c.len[1], D == 2 ? 1 : c.len[2]));
-  };
-  // ||T^-1||_inf of a line of n rows: |T^-1| is the inverse with off-diagonals
-  // -|b|, and its row sums solve that system for a right-hand side of ones;
-  // *grow: bound of the forward sweep for |g| <= 1
-  auto line_norm = [&](const Line& r, int n, double* grow) {
-    std::vector<double> v(n);
-    double u = 0.0, norm = 0.0;
-    for (int i = 0; i < n; ++i) {
-      v[i] = u = 1.0 + r.ld_[i] * u;
-      *grow = std::max(*grow, u);
-    }
-    for (int i = n - 1; i >= 0; --i) {
-      v[i] = (v[i] + (i + 1 < n ? r.b * v[i + 1] : 0.0)) * r.wd[i];
-      norm = std::max(norm, v[i]);
-    }
-    return norm;
-  };
   double t1 = 1.0, grow = 1.0, norm = 1.0;
   std::vector<std::vector<double>> norms(L.classes.size());
   for (size_t q = 0; q < L.classes.size(); ++q) {
     const RasClass& c = L.classes[q];
-    for (const Line& r : lines_of(c)) {
-      norms[q].push_back(line_norm(r, c.len[0], &grow));
+    const FixLines& ln = lines_of(c);
+    for (size_t sys = 0; sys < ln.b.size(); ++sys) {
+      norms[q].push_back(fix_line_norm(&ln.ld[sys * LM], &ln.wd[sys * LM], ln.b[sys], c.len[0], &grow));
       norm = std::max(norm, norms[q].back());
     }
-    for (int ax = 1; ax < D; ++ax) t1 = std::max(t1, ext[c.len[ax]].row);
+    for (int ax = 1; ax < D; ++ax) t1 = std::max(t1, ext.at(c.len[ax]).row);
   }
   // Quantisation: every operand of a multiply-add stays 1% below 2^60.
   // g bits of residual allow the fold (2), the transforms (t1 per axis), the
@@ -398,7 +482,7 @@ int ras_fix_setup(dcg_problem* p, Level& L, cudaStream_t s) {
     L.fx_kout = std::max(0, k3 - 1);
   }
   for (size_t q = 0; q < L.classes.size(); ++q) {
-    const Ext& ey = ext[L.classes[q].len[1]];
+    const FixExtent& ey = ext.at(L.classes[q].len[1]);
     for (double nr : norms[q]) {
       int k = k3;
       if (D == 2) {
@@ -410,7 +494,7 @@ int ras_fix_setup(dcg_problem* p, Level& L, cudaStream_t s) {
     }
   }
   L.fx_rb = std::min(L.fx_gb, 57);  // 6 r as an operand: at most 2^(fx_rb + 2)
-  L.fx_sixth = fx_const(fx_const_bits(1.0L / 6.0L));
+  L.fx_sixth = fx_const(fx_const_bits(dd_inverse(Dd{6.0, 0.0})));
 
   std::vector<int2> tab;
   for (size_t q = 0; q < L.classes.size(); ++q) {
@@ -418,7 +502,7 @@ int ras_fix_setup(dcg_problem* p, Level& L, cudaStream_t s) {
     const int2 none = make_int2(0, 0);
     for (int ax = 0; ax < D - 1; ++ax) {
       const int l = c.len[ax + 1], hc = (l + 1) / 2;
-      const std::vector<long long>& S = ext[l].S;
+      const std::vector<long long>& S = ext.at(l).S;
       if (tab.size() & 1) tab.push_back(none);  // the transforms' tables are read as 16-byte pairs
       c.fx_f[ax] = (int)tab.size();
       for (int j = 0; j < LM; ++j)
@@ -436,21 +520,21 @@ int ras_fix_setup(dcg_problem* p, Level& L, cudaStream_t s) {
           }
     }
     c.fx_tri = (int)tab.size();
-    const std::vector<Line>& ln = lines_of(c);
-    const int n = c.len[0], nsys = (int)ln.size();
+    const FixLines& ln = lines_of(c);
+    const int n = c.len[0], nsys = (int)ln.b.size();
     for (int sys = 0; sys < nsys; ++sys)
       if (!(norms[q][sys] * std::ldexp(1.0, -K[q][sys]) < 2.0)) {
         set_error_msg("fixed-point smoother: line factor out of range");
         return DCG_ERR_UNSUPPORTED;
       }
     for (int i = 0; i < n; ++i)
-      for (int sys = 0; sys < nsys; ++sys) tab.push_back(fx_const(ln[sys].l[i]));
+      for (int sys = 0; sys < nsys; ++sys) tab.push_back(fx_const(ln.l[(size_t)sys * LM + i]));
     for (int i = 0; i < n; ++i)
-      for (int sys = 0; sys < nsys; ++sys) tab.push_back(fx_const(ln[sys].w[i], -K[q][sys]));
+      for (int sys = 0; sys < nsys; ++sys) tab.push_back(fx_const(ln.w[(size_t)sys * LM + i], -K[q][sys]));
     for (int i = 0; i < n; ++i)
-      for (int sys = 0; sys < nsys; ++sys) tab.push_back(fx_const(ln[sys].bw[i]));
-    for (int sys = 0; sys < nsys; ++sys)
-      tab.push_back(n % 2 == 0 ? fx_const(ln[sys].meet[n / 2 - 1], -K[q][sys]) : none);
+      for (int sys = 0; sys < nsys; ++sys) tab.push_back(fx_const(ln.bw[(size_t)sys * LM + i]));
+    // read by lines of LM rows only
+    for (int sys = 0; sys < nsys; ++sys) tab.push_back(n == LM ? fx_const(ln.meet[sys], -K[q][sys]) : none);
   }
   L.fx_ntab = (int)tab.size();
   DCG_CUDA(cudaMalloc(&L.d_fix, sizeof(int2) * tab.size()));

@@ -628,11 +628,8 @@ struct SmallState {
   SmArgs args{};
   int lm = 0, ctas = kSmCtas;
   size_t smem = 0;
-  int* ops = nullptr;
-  int* boxes = nullptr;    // [2] per box of every smoothed level
-  double* tri = nullptr;   // [2 m^2 + m]
-  double* red = nullptr;   // [2 * kSmCtas]
-  int* ncyc = nullptr;
+  double* buf = nullptr;   // tri [2 m^2 + m], red [2 * kSmCtas], then the integers
+  std::vector<int> host;   // ops, boxes ([2] per box of every smoothed level), ncyc
 };
 
 // Algorithm 4 on level index k (0 = coarsest); levels up to `solo` are one
@@ -747,11 +744,7 @@ bool small_mg_supported(const dcg_problem* p) {
 void small_mg_free(dcg_problem* p) {
   SmallState* S = static_cast<SmallState*>(p->mg.small);
   if (!S) return;
-  cudaFree(S->ops);
-  cudaFree(S->boxes);
-  cudaFree(S->tri);
-  cudaFree(S->red);
-  cudaFree(S->ncyc);
+  cudaFree(S->buf);
   delete S;
   p->mg.small = nullptr;
 }
@@ -776,12 +769,9 @@ int small_mg_setup(dcg_problem* p, cudaStream_t s) {
   std::vector<size_t> box_end(J, 0);
   for (int k = 1; k < J; ++k) {
     const Level& L = p->levels[k];
-    std::vector<int> work(3 * (size_t)L.nwork);
-    DCG_CUDA(cudaMemcpyAsync(work.data(), L.d_work, sizeof(int) * work.size(), cudaMemcpyDeviceToHost, s));
-    DCG_CUDA(cudaStreamSynchronize(s));
     bpw[k] = L.npatch <= kSmCtas * warps ? 1 : 32 / group;
     for (int w = 0; w < L.nwork; ++w) {
-      const int cnt = work[3 * (size_t)w + 2];
+      const int cnt = L.item_count[w];
       for (int b = 0; b < (cnt + bpw[k] - 1) / bpw[k] * bpw[k]; ++b) {
         boxes.push_back(b < cnt ? w : -1);
         boxes.push_back(b);
@@ -789,9 +779,6 @@ int small_mg_setup(dcg_problem* p, cudaStream_t s) {
     }
     box_end[k] = boxes.size();
   }
-  DCG_CUDA(cudaMalloc(&S->boxes, sizeof(int) * boxes.size()));
-  DCG_CUDA(cudaMemcpyAsync(S->boxes, boxes.data(), sizeof(int) * boxes.size(), cudaMemcpyHostToDevice, s));
-  DCG_CUDA(cudaStreamSynchronize(s));  // the host list goes out of scope
   // solo levels: at most one box per warp of a CTA (a step takes 5,300 clocks
   // against 9,100 with cluster barriers; 15,000 in three rounds), and a coarsest
   // level of at most 15 per axis; with all levels solo one CTA does the solve
@@ -845,7 +832,6 @@ int small_mg_setup(dcg_problem* p, cudaStream_t s) {
     l.nclass = L.nclass;
     const int each = ctas_of(k) * warps;
     l.nbox = (int)(box_end[k] - box_end[k - 1]) / 2;
-    l.boxes = S->boxes + box_end[k - 1];
     l.bpw = bpw[k];
     l.rounds = (l.nbox / l.bpw + each - 1) / each;
     l.o_desc = take(sizeof(int4) * l.rounds * warps * l.bpw);
@@ -875,21 +861,6 @@ int small_mg_setup(dcg_problem* p, cudaStream_t s) {
     if (a.solo > 0 && a.solo < J - 1) sm_cycle(ops, p->opts, a.solo, false, -1);
   }
   a.nsolo = (int)ops.size() - a.nops;
-  DCG_CUDA(cudaMalloc(&S->ops, sizeof(int) * ops.size()));
-  DCG_CUDA(cudaMalloc(&S->tri, sizeof(double) * (2 * (size_t)m0 * m0 + m0)));
-  DCG_CUDA(cudaMalloc(&S->red, sizeof(double) * 2 * kSmCtas));
-  DCG_CUDA(cudaMalloc(&S->ncyc, sizeof(int)));
-  DCG_CUDA(cudaMemcpyAsync(S->ops, ops.data(), sizeof(int) * ops.size(), cudaMemcpyHostToDevice, s));
-  k_small_tri<<<(m0 + 63) / 64, 64, 0, s>>>(m0, S->tri, S->tri + (size_t)m0 * m0, S->tri + 2 * (size_t)m0 * m0);
-  DCG_LAUNCH_CHECK();
-  DCG_CUDA(cudaStreamSynchronize(s));  // the host list goes out of scope
-  a.ops = S->ops;
-  a.S = p->coarse.S64;
-  a.tl = S->tri;
-  a.tw = S->tri + (size_t)m0 * m0;
-  a.te = S->tri + 2 * (size_t)m0 * m0;
-  a.red = S->red;
-  a.ncyc = S->ncyc;
   bool fits = false;
   switch (S->lm) {
     case 4: DCG_TRY(sm_attr<4>(S->ctas, smem, &fits)); break;
@@ -899,7 +870,29 @@ int small_mg_setup(dcg_problem* p, cudaStream_t s) {
     case 12: DCG_TRY(sm_attr<12>(S->ctas, smem, &fits)); break;
     default: DCG_TRY(sm_attr<16>(S->ctas, smem, &fits));
   }
-  if (!fits) small_mg_free(p);  // the level-by-level kernels serve
+  if (!fits) {  // the level-by-level kernels serve
+    small_mg_free(p);
+    return DCG_OK;
+  }
+  // one buffer; the state keeps the host's copy of the integers, so the copy
+  // to the device needs no wait
+  const size_t ntri = 2 * (size_t)m0 * m0 + m0, ndbl = ntri + 2 * kSmCtas;
+  S->host = ops;
+  S->host.insert(S->host.end(), boxes.begin(), boxes.end());
+  S->host.push_back(0);
+  DCG_CUDA(cudaMalloc(&S->buf, sizeof(double) * ndbl + sizeof(int) * S->host.size()));
+  int* ints = reinterpret_cast<int*>(S->buf + ndbl);
+  DCG_CUDA(cudaMemcpyAsync(ints, S->host.data(), sizeof(int) * S->host.size(), cudaMemcpyHostToDevice, s));
+  k_small_tri<<<(m0 + 63) / 64, 64, 0, s>>>(m0, S->buf, S->buf + (size_t)m0 * m0, S->buf + 2 * (size_t)m0 * m0);
+  DCG_LAUNCH_CHECK();
+  a.ops = ints;
+  for (int k = 1; k < J; ++k) a.lev[k].boxes = ints + ops.size() + box_end[k - 1];
+  a.S = p->coarse.S64;
+  a.tl = S->buf;
+  a.tw = S->buf + (size_t)m0 * m0;
+  a.te = S->buf + 2 * (size_t)m0 * m0;
+  a.red = S->buf + ntri;
+  a.ncyc = ints + ops.size() + boxes.size();
   return DCG_OK;
 }
 
@@ -925,7 +918,7 @@ int small_mg_launch(dcg_problem* p, const double* g, double* z, bool fixed, doub
 int small_mg_cycles_done(dcg_problem* p, int* ncyc, cudaStream_t s) {
   SmallState* S = static_cast<SmallState*>(p->mg.small);
   int* host = reinterpret_cast<int*>(p->scal_host + S_COUNT - 1);  // pinned, unused slot
-  DCG_CUDA(cudaMemcpyAsync(host, S->ncyc, sizeof(int), cudaMemcpyDeviceToHost, s));
+  DCG_CUDA(cudaMemcpyAsync(host, S->args.ncyc, sizeof(int), cudaMemcpyDeviceToHost, s));
   DCG_CUDA(cudaStreamSynchronize(s));
   *ncyc = *host;
   return DCG_OK;
