@@ -379,7 +379,7 @@ int spmv_dot(dcg_problem* p, const double* x, double* y, const double* dv, int s
 int spmv_residual(dcg_problem* p, const double* f, const double* x, double* y, int slot, cudaStream_t s);
 // g = V^T A x, ||g||^2 into scal[slot]
 int spmv_vt(dcg_problem* p, const double* x, double* g, int slot, cudaStream_t s, bool lowp = false);
-// q = A (x - V zh) (zh may be null => x), dot(x, q) into scal[slot]; if x null: q = A (V zh)
+// q = A (x - V zh) (zh may be null => x), dot(x, q) into scal[slot]
 int spmv_defl(dcg_problem* p, const double* x, const double* zh, double* q, int slot, cudaStream_t s,
               bool lowp = false);
 // y = f - A(V zh), ||y||^2 into scal[slot]
@@ -392,8 +392,8 @@ int q_from_t(dcg_problem* p, const double* t, const double* zh, const double* dv
 // divergence stencil G[p*3+q][offset] of the uniform Q1 mesh (d = 2, 3)
 void div_stencil(int d, int n, double (*gs)[27]);
 // FP64 product with A in factored form (op.cu): operand x, x - V zh (both) or
-// V zh (x null); output y, f - y (f), V^T y (vt), or y and g = V^T y (g);
-// slot >= 0: dot (dvec, y), or the sum of squares of f - y, V^T y or g
+// V zh (x null, with f or vt); output y, f - y (f), V^T y (vt), or y and g = V^T y (g);
+// slot: dot (dvec, y), or the sum of squares of f - y, V^T y or g (y = A x alone: may be < 0)
 struct OpCall {
   const double* x = nullptr;
   const double* zh = nullptr;

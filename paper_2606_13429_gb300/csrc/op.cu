@@ -593,9 +593,10 @@ int op_time_rhs(dcg_problem* p, bool minus_div, const double* w, const double* f
   return op_launch<OX_X, OO_RHS, false>(p, a, s);
 }
 
-// y = A x in FP64. Operand x (zh null), x - V zh, or V zh (x null); output y,
-// f - y (f given), V^T y (vt), or y and g = V^T y (g given). slot >= 0: the sum
-// of squares of the output (of g when it is formed), or with dvec (dvec, y).
+// y = A x in FP64. Operand x (zh null), x - V zh, or V zh (x null, with f or vt);
+// output y, f - y (f given), V^T y (vt), or y and g = V^T y (g given). slot: the sum
+// of squares of the output (of g when it is formed), or with dvec (dvec, y);
+// y = A x alone may go without (slot < 0).
 int op_product(dcg_problem* p, const OpCall& c, cudaStream_t s) {
   OpArgs a = op_args(p, c);
   if (c.slot >= 0) a.red = make_reduce(p, c.slot);
@@ -608,24 +609,20 @@ int op_product(dcg_problem* p, const OpCall& c, cudaStream_t s) {
   double bytes = 8.0 * ((c.x ? N : 0.0) + (c.zh ? nn : 0.0) + (c.vt ? nn : N) + (c.g ? nn : 0.0) + (c.f ? N : 0.0) +
                         (c.dvec && c.dvec != c.x ? N : 0.0) + (a.inv_nu ? nn : 0.0));
   const int prof = prof_begin(p, PC_SPMV, s);
-  const bool dot = c.slot >= 0;
-  int st = DCG_ERR_UNSUPPORTED;
-#define DCG_OP(XMV, OMV) st = dot ? op_launch<XMV, OMV, true>(p, a, s) : op_launch<XMV, OMV, false>(p, a, s)
+  int st;
   if (c.x && !c.zh) {
-    if (c.vt) DCG_OP(OX_X, OO_VT);
-    else if (c.g) DCG_OP(OX_X, OO_YVT);
-    else if (c.f) DCG_OP(OX_X, OO_FMY);
-    else DCG_OP(OX_X, OO_Y);
+    if (c.vt) st = op_launch<OX_X, OO_VT, true>(p, a, s);
+    else if (c.g) st = op_launch<OX_X, OO_YVT, true>(p, a, s);
+    else if (c.f) st = op_launch<OX_X, OO_FMY, true>(p, a, s);
+    else if (c.slot >= 0) st = op_launch<OX_X, OO_Y, true>(p, a, s);
+    else st = op_launch<OX_X, OO_Y, false>(p, a, s);
   } else if (c.x) {
     st = op_launch<OX_X_MINUS_VZ, OO_Y, true>(p, a, s);
   } else if (c.vt) {
     st = op_launch<OX_VZ, OO_VT, true>(p, a, s);
-  } else if (c.f) {
-    st = op_launch<OX_VZ, OO_FMY, true>(p, a, s);
   } else {
-    st = op_launch<OX_VZ, OO_Y, false>(p, a, s);
+    st = op_launch<OX_VZ, OO_FMY, true>(p, a, s);
   }
-#undef DCG_OP
   DCG_TRY(st);
   prof_end(p, prof, s, 2.0 * ops * nn, bytes);
   return DCG_OK;

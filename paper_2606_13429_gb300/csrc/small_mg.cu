@@ -35,7 +35,7 @@ namespace {
 
 constexpr int kSmCtas = 16;     // CTAs of the cluster
 constexpr int kSmLevels = 8;
-constexpr int sm_threads(int LM) { return 512; }
+constexpr int kSmThreads = 512;
 // shared memory of one box: z with its halo, and two copies of the box values
 constexpr int sm_box_words(int LM) { return (LM + 2) * (LM + 2) + 2 * LM * (LM | 1); }
 
@@ -132,7 +132,7 @@ __device__ __forceinline__ double sm_residual(double c0, double c1, double fv, c
 // and the offset of the box's results in y.
 template <int LM>
 __device__ __forceinline__ void sm_stage(const SmLevel& L, int rank, int ctas, unsigned char* smem) {
-  constexpr int NT = sm_threads(LM), NW = NT / 32;
+  constexpr int NT = kSmThreads, NW = NT / 32;
   if (L.o_tab >= 0)
     for (int t = threadIdx.x; t < L.ntab; t += NT) reinterpret_cast<int2*>(smem + L.o_tab)[t] = __ldg(L.tab + t);
   for (int t = threadIdx.x; t < L.nclass; t += NT) {
@@ -275,7 +275,7 @@ __device__ __forceinline__ void sm_box(const FxScale& sc, bool zzero, int lx, in
 template <int LM, bool SOLO>
 __device__ __forceinline__ void sm_ras(const SmLevel& L, const SmVec& V, bool zzero, int restricted, int rank, int ctas,
                                        unsigned char* smem, int o_work) {
-  constexpr int NT = sm_threads(LM), NW = NT / 32;
+  constexpr int NT = kSmThreads, NW = NT / 32;
   const int warp = threadIdx.x >> 5;
   const int4* desc = reinterpret_cast<const int4*>(smem + L.o_desc);
   const int2* tab = L.o_tab >= 0 ? reinterpret_cast<const int2*>(smem + L.o_tab) : L.tab;
@@ -468,7 +468,7 @@ __device__ __forceinline__ void sm_coarse(const SmArgs& A, const double* S, cons
 template <int LM, bool SOLO>
 __device__ __forceinline__ void sm_run(const SmArgs& A, int op, const double* S, int rank, int ctas,
                                        unsigned char* smem) {
-  constexpr int NT = sm_threads(LM);
+  constexpr int NT = kSmThreads;
   const int kind = op & 255, k = op >> 8;
   const SmLevel& L = A.lev[k];
   double* work = reinterpret_cast<double*>(smem + A.o_work);
@@ -521,8 +521,8 @@ __device__ __noinline__ double sm_to_one(double* f, int nn, double* red, int ran
 }
 
 template <int LM>
-__global__ void __launch_bounds__(sm_threads(LM), 1) k_small_mg(const __grid_constant__ SmArgs A) {
-  constexpr int NT = sm_threads(LM);
+__global__ void __launch_bounds__(kSmThreads, 1) k_small_mg(const __grid_constant__ SmArgs A) {
+  constexpr int NT = kSmThreads;
   extern __shared__ __align__(16) unsigned char sm_smem[];
   __shared__ double s_red[64];
   const int rank = blockIdx.x, ctas = gridDim.x;  // one cluster, or one CTA
@@ -679,7 +679,7 @@ int sm_attr(int ctas, size_t smem, bool* fits) {
   DCG_CUDA(cudaFuncSetAttribute(k_small_mg<LM>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute at[1];
-  sm_config(ctas, sm_threads(LM), smem, nullptr, &cfg, at);
+  sm_config(ctas, kSmThreads, smem, nullptr, &cfg, at);
   int n = 0;
   if (cudaOccupancyMaxActiveClusters(&n, k_small_mg<LM>, &cfg) != cudaSuccess) {
     cudaGetLastError();
@@ -693,7 +693,7 @@ template <int LM>
 cudaError_t sm_start(const SmArgs& a, int ctas, size_t smem, cudaStream_t s) {
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute at[1];
-  sm_config(ctas, sm_threads(LM), smem, s, &cfg, at);
+  sm_config(ctas, kSmThreads, smem, s, &cfg, at);
   return cudaLaunchKernelEx(&cfg, k_small_mg<LM>, a);
 }
 
@@ -760,7 +760,7 @@ int small_mg_setup(dcg_problem* p, cudaStream_t s) {
   S->lm = ras_fix_lm(2, p->levels.back().fdm_lmax);
   a.nlev = J;
   a.restricted = p->opts.ras_weights == DCG_RAS_RESTRICTED;
-  const int nt = sm_threads(S->lm), warps = nt / 32;
+  const int nt = kSmThreads, warps = nt / 32;
   // The levels' boxes in the order of their work items: one per warp where the
   // cluster has a warp for each, else in groups of one class (a lane per
   // column; 95^2: 11,000 clocks per step against 18,300 in three rounds).

@@ -6,7 +6,7 @@
 // Variants (x operand / output):
 //   x            : y = A x
 //   x - V zh     : q = A (d - V zh)          (M_D of Algorithm 2, second product)
-//   V zh         : y = A V zh                 (A pi(f) for f_D)
+//   V zh         : f - A V zh                 (f_D = f - A pi(f))
 //   out = y / f - y / V^T y / y and V^T y.
 #include "common.cuh"
 
@@ -32,7 +32,7 @@ namespace {
 // Variants (x operand / output):
 //   x            : y = A x
 //   x - V zh     : q = A (d - V zh)          (M_D of Algorithm 2, second product)
-//   V zh         : y = A V zh                 (A pi(f) for f_D)
+//   V zh         : f - A V zh                 (f_D = f - A pi(f))
 //   out = y / f - y / V^T y (only the d diagonal-component rows are computed:
 //   g = V^T A x reads half (2D) or a third (3D) of the matrix).
 enum XMode { XM_X = 0, XM_X_MINUS_VZ = 1, XM_VZ = 2 };
@@ -323,7 +323,7 @@ int bsr_product(dcg_problem* p, const OpCall& c, cudaStream_t s) {
   a.g = c.g;
   a.dvec = c.dvec;
   if (c.slot >= 0) a.red = make_reduce(p, c.slot);
-  if (!c.x) return c.f ? launch<XM_VZ, OM_FMY, true>(p, a, s) : launch<XM_VZ, OM_Y, false>(p, a, s);
+  if (!c.x) return launch<XM_VZ, OM_FMY, true>(p, a, s);
   if (c.zh) return launch<XM_X_MINUS_VZ, OM_Y, true>(p, a, s);
   if (c.vt) return launch<XM_X, OM_VT, true>(p, a, s);
   if (c.f) return launch<XM_X, OM_FMY, true>(p, a, s);
@@ -382,16 +382,14 @@ int spmv_vt(dcg_problem* p, const double* x, double* g, int slot, cudaStream_t s
 }
 
 int spmv_defl(dcg_problem* p, const double* x, const double* zh, double* q, int slot, cudaStream_t s, bool lowp) {
-  if (x && lowp && p->matrix_free)
+  if (lowp && p->matrix_free)
     return mf_product(p, zh ? 1 : 0, 0, true, x, zh, q, x, make_reduce(p, slot), s);
   OpCall c;
   c.x = x;
   c.zh = zh;
   c.y = q;
-  if (x) {
-    c.dvec = x;
-    c.slot = slot;
-  }
+  c.dvec = x;
+  c.slot = slot;
   return product(p, c, s);
 }
 
