@@ -478,8 +478,9 @@ def run_ours(args):
             "config": {"workload": WORKLOAD, "parallelism": "replicas" if ws > 1 else "single GPU",
                        "mg_levels": best_levels, "dts": DTS,
                        "value": "mean over the six dt of the time to solution (each dt the mean of its timed steps)",
-                       "smoother": "RAS, FP64 local solves by fast diagonalisation (sine transforms + line solves)",
-                       "l2": "inputs larger than L2 (BSR matrix 1.2 GB per dt, 6 matrices)",
+                       "smoother": "RAS, exact local solves by fast diagonalisation (sine transforms + line solves) in "
+                                   "64-bit fixed point (53 to 58 bits of a box's largest entry)",
+                       "l2": "working set larger than L2 (solver vectors 0.23 GB; the products read no stored blocks)",
                        "all_converged": ok},
             "e2e": {"value": e2e_s, "unit": "s/solve", "h2d_bytes_per_step": 2 * N * 8, "d2h_bytes_per_step": N * 8,
                     "steps": len(DTS), "note": "one sweep (each dt once) through dcg_solve_host"},

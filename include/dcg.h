@@ -77,7 +77,10 @@ extern "C" {
                            length fcg_max_dirs, inner tolerance of Eq. tol from the
                            least-squares residual norm; host-driven loop */
 
-#define DCG_FP64   0  /* everything in FP64 */
+#define DCG_FP64   0  /* everything in FP64 but the exact box solves of the RAS smoother, which
+                         run in 64-bit fixed point: errors relative to the largest entry of a
+                         box, which has 55 to 58 bits (2D steps from a nonzero iterate: 53 to 56
+                         bits of the residual, formed exactly from z and f), against FP64's 53 */
 #define DCG_MIXED  1  /* W-cycle (stencils, transfers, RAS) in FP32; outer CG FP64 */
 
 #define DCG_INV_FP32  0  /* RAS patch inverses stored FP32 (mixed mode) */

@@ -15,10 +15,13 @@
 // L2 round trip (with them in global memory a phase took 3.1 us).
 //
 // The smoother is the box solve of ras_fix.cuh, a warp per box, with the work
-// items, tables and box results of the level's own kernels; residuals, transfers and weighted sums use the same expressions,
-// so one smoothing step or transfer gives the same bits as the kernels of
-// mg.cu. The coarsest level is solved by dense sine passes around Thomas
-// line solves, its rows and lines spread over the CTAs.
+// items, tables and box results of the level's own kernels; residuals, transfers
+// and weighted sums use the same expressions. A step agrees with the kernels of
+// mg.cu to rounding: lines of the largest extent are eliminated from both ends,
+// there only in boxes that have it along every axis, here in every such line,
+// and in groups of boxes from a zero iterate in none. The coarsest level is
+// solved by dense sine passes around Thomas line solves, its rows and lines
+// spread over the CTAs.
 //
 // Measured per inner solve (relative tolerance 1e-10, about 5 cycles), level-by-level
 // kernels with the FP64 smoother against this form: four levels, 4 x 4
@@ -155,9 +158,8 @@ __device__ __forceinline__ void sm_stage(const SmLevel& L, int rank, int ctas, u
       reinterpret_cast<int4*>(smem + L.o_ysrc)[k] = __ldg(reinterpret_cast<const int4*>(L.ysrc) + a);
 }
 
-// Exact solve on one box by one warp: the arithmetic of fx_solve_2d (the same
-// integers, so the same bits), with the entries of every stage spread over
-// the 32 lanes. A lone warp is latency bound, about six clocks per
+// Exact solve on one box by one warp: the arithmetic of fx_solve_2d, with the
+// entries of every stage spread over the 32 lanes. A lone warp is latency bound, about six clocks per
 // instruction, so the count per lane is what a small level costs: with a lane
 // per column a step's solve took 5,700 clocks whatever the level's size.
 template <int LM, bool SOLO>
@@ -720,16 +722,21 @@ int sm_dispatch(const SmallState& S, const SmArgs& a, cudaStream_t s) {
 
 // The one-kernel solve serves FP64 2D hierarchies of at least two levels whose
 // smoothed levels are box-sum levels with fixed-point local solves, with at
-// most kSmallNodes nodes on the finest level (two levels: kSmallNodes2) and 80 per axis on the coarsest
-// (its dense passes grow with the cube). Per inner solve against the
-// level-by-level kernels with fixed-point smoother, us: four levels, 4 x 4
-// cores, 112^2 1,171 / 1,664, 160^2 1,428 / 1,733; two levels, 4 x 4 cores, 64^2
-// 324 / 428, 112^2 428 / 503, 128^2 503 / 467, 160^2 630 / 569; 8 x 8 cores, 128^2
-// 543 / 568, 160^2 675 / 679. Above these sizes a phase no longer is the
-// latency of one round, with two levels sooner (fewer phases per cycle, more
-// work in each): whole captured solves of two levels, 4 x 4 cores, take 8.18
-// against 6.64 ms at 128^2 and 12.22 against 10.02 at 160^2, so two levels stop
-// at kSmallNodes2.
+// most kSmallNodes nodes on the finest level (two levels: kSmallNodes2) and 80
+// per axis on the coarsest (its dense passes grow with the cube). Per inner
+// solve against the level-by-level kernels with fixed-point smoother, us: four
+// levels, 4 x 4 cores, 112^2 1,171 / 1,664, 160^2 1,428 / 1,733; two levels, 4 x 4
+// cores, 64^2 324 / 428, 112^2 428 / 503, 128^2 503 / 467, 160^2 630 / 569; 8 x 8
+// cores, 128^2 543 / 568, 160^2 675 / 679. Above these sizes a phase no longer is
+// the latency of one round, with two levels sooner (fewer phases per cycle,
+// more work in each): whole captured solves of two levels, 4 x 4 cores, take
+// 8.18 against 6.64 ms at 128^2 and 12.22 against 10.02 at 160^2, so two levels
+// stop at kSmallNodes2. Deeper hierarchies stop at the largest size measured;
+// their crossing lies above it.
+// A solve holds 16 SMs, so about nine run at a time, the level kernels of a
+// batch more; batches gain all the same (ms, one kernel / level kernels): 64
+// problems, two levels 32^2 67 / 103, 112^2 77 / 114, four levels 32^2 152 / 408,
+// 112^2 197 / 357; 8 problems, two levels 112^2 10.0 / 14.3.
 constexpr long long kSmallNodes = 26000, kSmallNodes2 = 13000;
 bool small_mg_supported(const dcg_problem* p) {
   const int J = (int)p->levels.size();

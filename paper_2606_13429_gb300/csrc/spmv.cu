@@ -307,7 +307,9 @@ int launch(dcg_problem* p, SpmvArgs a, cudaStream_t s) {
 // Measured, uniform viscosity / one per element (us): 2D 95^2 6.8 / 8.2
 // against 5.0, 179^2 11.8 / 15.3 against 10.5, 256^2 11.8 / 15.4 against 18.6;
 // 3D 15^3 13.6 / 20.5 against 10.1, 19^3 13.7 / 20.6 against 19.3, 23^3 16.7 /
-// 25.3 against 39.5.
+// 25.3 against 39.5. One line serves both: with a viscosity per element the
+// blocks are still ahead at 19^3 (6,859 nodes), where a uniform one gives 5.6 us
+// away by it.
 // The 2D kernel reads x as 16-byte pairs: an operand that is only 8-byte
 // aligned goes to the factored product, which checks.
 bool bsr_better(const dcg_problem* p, const OpCall& c) {
