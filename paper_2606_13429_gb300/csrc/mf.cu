@@ -22,6 +22,12 @@
 // grid) in shared memory, one array per component; each thread produces one
 // node per plane. Input and output stay FP64 in memory (the FP64 product is
 // op.cu's).
+//
+// What bounds it (1.61 ms at 256^3, 0.37 ms of memory traffic): no single unit.
+// The FP64 pipe is the busiest, 56%, with the conversions of operands (1.33 per
+// entry with the halo) and results; issue slots are 56% busy, shared-memory
+// wavefronts 26%. A plane is loaded and converted right before the barrier that
+// precedes its use, which exposes the latency.
 #include "common.cuh"
 
 namespace dcg {
